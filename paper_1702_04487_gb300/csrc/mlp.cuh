@@ -62,8 +62,8 @@ struct Xform {
 };
 
 // Raw rows x [n][7] -> transformed BF16 rows X [n][16] (columns 7.. zero)
-// and FP32 transformed copy Xf [n][7] (either may be null).
-cudaError_t launch_prep_inputs(const float* x, int n, const Xform& xf, bf16* X, float* Xf,
+// and FP32 transformed columns Xf [7][ldx] (either may be null).
+cudaError_t launch_prep_inputs(const float* x, int n, const Xform& xf, bf16* X, float* Xf, int ldx,
                                cudaStream_t s);
 // Raw targets y [n][4] -> transformed FP32 T [n][4].
 cudaError_t launch_prep_targets(const float* y, int n, const Xform& yf, float* T, cudaStream_t s);
@@ -105,17 +105,35 @@ cudaError_t launch_schedule_begin(const long long* d_step, long long* d_sched, l
 cudaError_t launch_cast_params(const float* p, const Layout& L, int members, bf16* Wb, bf16* WbT,
                                cudaStream_t s);
 cudaError_t launch_advance_step(long long* d_step, cudaStream_t s);
-// Member outputs Y [m][n][16] -> inverse-transformed outcomes, their mean
-// and standard deviation over members: mean [n][4], std [n][4].
-cudaError_t launch_decode(const float* Y, int n, int members, const Xform& yf, float* mean,
-                          float* sd, cudaStream_t s);
-// Acceptance gate: inside the per-feature box [lo, hi] of the training
-// inputs, nearest training point (transformed space) within nn_cut, and
-// relative ensemble spread sd/|mean| of outcome 0 below tau and of
-// outcome 1 below tau_v.
-cudaError_t launch_gate(const float* x, const float* Xq, int n, const float* Xtrain, int nt,
-                        const float* lo, const float* hi, float nn_cut, const float* mean,
-                        const float* sd, float tau, float tau_v, int* accept, float* nn_dist,
-                        cudaStream_t s);
+// Outputs of every member for n raw queries x [n][7]: Y [m][n][4] (FP32,
+// transformed outcomes).  One kernel runs all five layers of a 128-row tile.
+cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* p, const bf16* Wb,
+                           const Layout& L, int members, float* Y, unsigned* status,
+                           cudaStream_t s);
+
+// The answers of n queries from the member outputs Y [m][n][4]: the mean
+// [n][4] and standard deviation [n][4] over members of the inverse-
+// transformed outcomes, and (accept not null) the acceptance gate: inside
+// the per-feature box [lo, hi] of the training inputs, within nn_cut of a
+// training point (transformed space; Xt [7][ldt], nt points), and relative
+// ensemble spread sd/|mean| of outcome 0 at most tau and of outcome 1 at
+// most tau_v.  *status_out receives *status.
+struct GateArgs {
+  const float* x;
+  const float* Y;
+  int n, members;
+  Xform xin, xout;
+  const float* Xt;
+  int nt, ldt;
+  const float* lo;
+  const float* hi;
+  float nn_cut, tau, tau_v;
+  float* mean;
+  float* sd;
+  int* accept;
+  const unsigned* status;
+  unsigned* status_out;
+};
+cudaError_t launch_answer(const GateArgs& a, cudaStream_t s);
 
 }  // namespace sg

@@ -410,14 +410,14 @@ __device__ __forceinline__ float xform(float v, int d, const Xform& xf) {
 }
 
 __global__ void prep_inputs_kernel(const float* __restrict__ x, int n, const Xform xf,
-                                   bf16* __restrict__ X, float* __restrict__ Xf) {
+                                   bf16* __restrict__ X, float* __restrict__ Xf, int ldx) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
 #pragma unroll
   for (int d = 0; d < kInPad; d++) {
     const float v = d < kIn ? xform(x[(size_t)r * kIn + d], d, xf) : 0.0f;
     if (X) X[(size_t)r * kInPad + d] = __float2bfloat16_rn(v);
-    if (Xf && d < kIn) Xf[(size_t)r * kIn + d] = v;
+    if (Xf && d < kIn) Xf[(size_t)d * ldx + r] = v;
   }
 }
 
@@ -575,81 +575,340 @@ __global__ void cast_params_kernel(const float* __restrict__ p, const Layout L, 
 
 __global__ void advance_step_kernel(long long* d_step) { *d_step += 1; }
 
-__global__ void decode_kernel(const float* __restrict__ Y, int n, int members, const Xform yf,
-                              float* __restrict__ mean, float* __restrict__ sd) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
+// ---------------------------------------------------------------------------
+// Inference: all five layers of a 128-row tile of queries for one member in
+// one CTA.  The tile's activations stay in shared memory (BF16, the K-major
+// 128-byte-swizzled layout the tensor cores read) and the accumulator in
+// tensor memory; only the queries are read and the four outcomes written, so
+// nothing of a hidden layer touches HBM.  Weights stream from L2 through a
+// ring of 64 (K) x 128 (output units) chunks loaded by the tensor memory
+// accelerator; they do not depend on the activations, so the chunks of the
+// next layer are fetched while this layer's outputs are computed.  Thread 0
+// loads and issues; the output pass of a hidden layer (bias, GELU, rounding
+// to BF16, swizzled 16-byte stores) is shared by every warp: warp w reads
+// tensor-memory lanes 32 (w mod 4) .. + 31 and every (warps / 4)-th group of
+// 16 units.
+//
+// Bound by the GELUs (an erff each: 4 H per query and member) at instruction
+// issue; two CTAs of 256 threads share an SM, so one's tensor-core pass and
+// weight loads run beside the other's GELUs.  While the grid has at most one
+// tile per SM, one CTA of 512 threads and a ring of nine chunks per SM halve
+// the serial chain of a layer instead.  Measured, five members of H = 256:
+// 65536 queries 500 us, against 2190 us for a GEMM launch per layer with the
+// activations through HBM (the same results, bit for bit).
+constexpr int kFwdChunk = 128 * BK * 2;  // bytes of a weight chunk, and of 64 activation columns
+constexpr int kFwdRingMax = 9;
+
+struct FwdMaps {
+  CUtensorMap w[kHidden + 1];  // boxes of 64 (K) x 128 (units) x 1 (member)
+};
+struct FwdArgs {
+  const float* x;
+  int n, H;
+  Xform xf;
+  const float* p;
+  long long P;
+  int b_off[kHidden + 1];
+  float* Y;
+  unsigned* status;
+};
+
+template <int NT>
+__host__ __device__ constexpr int fwd_ring() {
+  return NT == 256 ? 3 : kFwdRingMax;
+}
+// activations, ring, then the barriers and the tensor-memory address (no
+// static shared memory: the dynamic part then starts on a 1024-byte boundary
+// and two CTAs of H = 256 fit an SM)
+constexpr int kFwdTail = 256;
+size_t fwd_smem_bytes(int H, int ring) {
+  return (size_t)((H + BK - 1) / BK + ring) * kFwdChunk + kFwdTail;
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
+    forward_kernel(const __grid_constant__ FwdMaps maps, const FwdArgs a) {
+  extern __shared__ __align__(1024) uint8_t fwd_smem[];
+  constexpr int R = fwd_ring<NT>();
+  const int H = a.H, slices = (H + BK - 1) / BK;
+  uint8_t* const smem = fwd_smem;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + (size_t)(slices + R) * kFwdChunk);
+  uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * R + 1);
+  static_assert((2 * R + 1) * 8 + 4 <= kFwdTail, "barriers outgrew their slot");
+  const uint32_t act = smem_u32(smem);
+  if (act & 1023u) {  // the swizzled layout needs the alignment asked for
+    if (threadIdx.x == 0) atomicOr(a.status, kStatusTimeout);
+    return;
+  }
+  const uint32_t ring = act + (uint32_t)slices * kFwdChunk;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.x * BM, z = blockIdx.y;
+  const uint32_t cols = H <= 32 ? 32 : H <= 64 ? 64 : H <= 128 ? 128 : 256;
+  // bars[b]: chunk landed; bars[R + b]: its MMAs done; bars[2 R]: layer done
+  if (tid == 0) {
 #pragma unroll
-  for (int d = 0; d < kOut; d++) {
-    double s = 0.0, s2 = 0.0;
-    for (int mem = 0; mem < members; mem++) {
-      float v = Y[((size_t)mem * n + q) * kOutPad + d] * yf.scale[d] + yf.mean[d];
-      if ((yf.log_mask >> d) & 1) v = expf(v);
-      s += v;
-      s2 += (double)v * v;
+    for (int i = 0; i < 2 * R + 1; i++) mbar_init(smem_u32(&bars[i]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+
+  // Chunk c of the member's weights, in the order they are used: layer by
+  // layer, K slice by K slice, 128 output units at a time.
+  int ld_l = 0, ld_s = 0, ld_h = 0, loaded = 0;  // the next chunk to load
+  auto units_of = [&](int l) { return l < kHidden ? H : kOutPad; };
+  auto depth_of = [&](int l) { return l == 0 ? kInPad : H; };
+  auto load_next = [&]() {
+    if (ld_l > kHidden) return;
+    const int b = loaded % R;
+    const uint32_t bar = smem_u32(&bars[b]);
+    mbar_expect_tx(bar, (uint32_t)kFwdChunk);
+    tma_load3(ring + (uint32_t)b * kFwdChunk, &maps.w[ld_l], ld_s * BK, ld_h * 128, z, bar);
+    loaded++;
+    if ((++ld_h) * 128 >= units_of(ld_l)) {
+      ld_h = 0;
+      if ((++ld_s) * BK >= depth_of(ld_l)) {
+        ld_s = 0;
+        ld_l++;
+      }
     }
-    const double mu = s / members;
-    mean[(size_t)q * kOut + d] = (float)mu;
-    sd[(size_t)q * kOut + d] = (float)sqrt(fmax(s2 / members - mu * mu, 0.0));
+  };
+  if (tid == 0)
+    for (int i = 0; i < R; i++) load_next();
+
+  // layer 0's operand: transformed queries, BF16, columns 7..15 zero
+  if (tid < BM) {
+    const int row = m0 + tid;
+    __align__(16) bf16 v[kInPad];
+#pragma unroll
+    for (int d = 0; d < kInPad; d++)
+      v[d] = __float2bfloat16_rn(
+          d < kIn && row < a.n ? xform(a.x[(size_t)row * kIn + d], d, a.xf) : 0.0f);
+#pragma unroll
+    for (int c = 0; c < 2; c++)
+      *reinterpret_cast<uint4*>(smem + tid * 128 + ((c ^ (tid & 7)) << 4)) =
+          reinterpret_cast<const uint4*>(v)[c];
+  }
+  const bool rows_in = m0 + (warp & 3) * 32 < a.n;  // any valid row of this warp's 32
+  uint32_t tmem = 0;
+  int used = 0, freed = 0;  // thread 0: chunks whose MMAs were issued / seen done
+  bool ok = true;
+  for (int l = 0; l <= kHidden; l++) {
+    // the operand written by every thread is visible to the tensor cores
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (l == 0) tmem = *(volatile uint32_t*)tmem_slot;
+    if (tid == 0) {
+      const int K = depth_of(l), N = units_of(l);
+      for (int s = 0; s * BK < K && ok; s++)
+        for (int h = 0; h * 128 < N && ok; h++) {
+          const int b = used % R;
+          if (!mbar_wait(smem_u32(&bars[b]), (uint32_t)((used / R) & 1))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const int nn = N - h * 128 < 128 ? N - h * 128 : 128;
+          const int steps = K - s * BK < BK ? (K - s * BK) / 16 : BK / 16;
+          const uint32_t ta = act + (uint32_t)s * kFwdChunk, tb = ring + (uint32_t)b * kFwdChunk;
+          const uint32_t id = idesc_bf16(BM, nn);
+          for (int k = 0; k < steps; k++)
+            mma_bf16(tmem + h * 128, sw128_desc(ta + 32 * k), sw128_desc(tb + 32 * k), id,
+                     (s > 0 || k > 0) ? 1u : 0u);
+          mma_commit(smem_u32(&bars[R + b]));
+          used++;
+          // refill the buffer of the chunk before once its MMAs are done
+          if (used >= 2 && ld_l <= kHidden && loaded < used - 1 + R) {
+            if (!mbar_wait(smem_u32(&bars[R + (used - 2) % R]), (uint32_t)(((used - 2) / R) & 1))) {
+              ok = false;
+              break;
+            }
+            freed = used - 1;
+            load_next();
+          }
+        }
+      if (ok) {
+        // an arrival once every MMA of the layer is done
+        mma_commit(smem_u32(&bars[2 * R]));
+        ok = mbar_wait(smem_u32(&bars[2 * R]), (uint32_t)(l & 1));
+        if (ok) {
+          freed = used;
+          while (ld_l <= kHidden && loaded < used + R) load_next();
+        }
+      }
+    }
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    tc_fence_after();
+    if (l < kHidden) {
+      const float* bias = a.p + z * a.P + a.b_off[l];
+      if (rows_in)
+#pragma unroll 1
+        for (int c0 = (warp >> 2) * 16; c0 < H; c0 += NT / 128 * 16) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+          __align__(16) bf16 o[16];
+#pragma unroll
+          for (int j = 0; j < 16; j++) o[j] = __float2bfloat16_rn(gelu_f(v[j] + __ldg(bias + c0 + j)));
+          const int r = (warp & 3) * 32 + lane, sl = c0 / BK, ch = (c0 % BK) / 8;
+          uint8_t* row = smem + (size_t)sl * kFwdChunk + r * 128;
+#pragma unroll
+          for (int c = 0; c < 2; c++)
+            *reinterpret_cast<uint4*>(row + (((ch + c) ^ (r & 7)) << 4)) =
+                reinterpret_cast<const uint4*>(o)[c];
+        }
+    } else if (warp < 4 && rows_in) {
+      float v[16];
+      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16), v);
+      const int row = m0 + warp * 32 + lane;
+      const float* bias = a.p + z * a.P + a.b_off[l];
+      if (row < a.n)
+        *reinterpret_cast<float4*>(a.Y + ((size_t)z * a.n + row) * kOut) =
+            make_float4(v[0] + __ldg(bias), v[1] + __ldg(bias + 1), v[2] + __ldg(bias + 2),
+                        v[3] + __ldg(bias + 3));
+    }
+  }
+  if (!ok) {
+    // no copy may land and no MMA run after the CTA gives up its memory
+    // (bounded again)
+    if (tid == 0) {
+      for (int c = used; c < loaded; c++) mbar_wait(smem_u32(&bars[c % R]), (uint32_t)((c / R) & 1));
+      for (int c = freed > used - R ? freed : used - R; c < used; c++)
+        if (c >= 0) mbar_wait(smem_u32(&bars[R + c % R]), (uint32_t)((c / R) & 1));
+      atomicOr(a.status, kStatusTimeout);
+    }
+    if (tmem == 0) tmem = *(volatile uint32_t*)tmem_slot;
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(cols)
+                 : "memory");
   }
 }
 
-constexpr int kGateTile = 512;
+// Answers of QB queries per block: a thread per (query, outcome) decodes and
+// reduces over the members; the queries that pass the box and spread tests
+// are listed, and warps look for a training point within nn_cut of them, a
+// lane per training point, four points in flight per lane, stopping at the
+// first hit (the gate asks whether the nearest point is within nn_cut, so any
+// point within it decides).  A short list gives each query several warps.
+//
+// Bound by the distance search (FP32 pipe and L1 loads of the points, laid
+// out by column so that a warp reads 128-byte lines).  One thread scanning
+// all points for its query took 194 us for one query and 220 us for 65536
+// against 4096 points (a serial chain of 4096 shared-memory reads per query),
+// and decoding another 10 to 28 us; now 10 and 37 us for both.
+constexpr int kAnswerThreads = 256;
+constexpr int kScan = 4;  // points in flight per lane
 
-__global__ void gate_kernel(const float* __restrict__ x, const float* __restrict__ Xq, int n,
-                            const float* __restrict__ Xtrain, int nt, const float* __restrict__ lo,
-                            const float* __restrict__ hi, float nn_cut,
-                            const float* __restrict__ mean, const float* __restrict__ sd,
-                            float tau, float tau_v, int* __restrict__ accept,
-                            float* __restrict__ nn_dist) {
-  __shared__ float tile[kGateTile * kIn];
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  float xq[kIn];
-  bool inbox = q < n;
-#pragma unroll
-  for (int d = 0; d < kIn; d++) {
-    xq[d] = q < n ? Xq[(size_t)q * kIn + d] : 0.0f;
-    if (q < n) {
-      const float raw = x[(size_t)q * kIn + d];
-      inbox = inbox && raw >= lo[d] && raw <= hi[d];
+template <int QB>
+__global__ void __launch_bounds__(kAnswerThreads) answer_kernel(const GateArgs a) {
+  constexpr int kWarps = kAnswerThreads / 32;
+  __shared__ int list[QB];
+  __shared__ int hit[QB];
+  __shared__ int count;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q0 = blockIdx.x * QB;
+  if (tid == 0) {
+    count = 0;
+    if (blockIdx.x == 0) *a.status_out = *(volatile const unsigned*)a.status;
+  }
+  __syncthreads();
+  // decode: the four outcomes of a query on four neighbouring lanes
+  for (int k = tid; k < QB * kOut; k += kAnswerThreads) {
+    const int q = q0 + (k >> 2), d = k & 3;
+    const bool in = q < a.n;
+    bool ok = in;
+    if (in) {
+      double s = 0.0, s2 = 0.0;
+      const float sc = a.xout.scale[d], mn = a.xout.mean[d];
+      const bool lg = (a.xout.log_mask >> d) & 1;
+      for (int mem = 0; mem < a.members; mem++) {
+        float v = a.Y[((size_t)mem * a.n + q) * kOut + d] * sc + mn;
+        if (lg) v = expf(v);
+        s += v;
+        s2 += (double)v * v;
+      }
+      const double mu = s / a.members;
+      const float muf = (float)mu, sdf = (float)sqrt(fmax(s2 / a.members - mu * mu, 0.0));
+      a.mean[(size_t)q * kOut + d] = muf;
+      a.sd[(size_t)q * kOut + d] = sdf;
+      if (d < 2) ok = isfinite(muf) && sdf <= (d == 0 ? a.tau : a.tau_v) * fabsf(muf);
+      if (a.accept)
+        for (int j = d; j < kIn; j += kOut) {
+          const float raw = a.x[(size_t)q * kIn + j];
+          ok = ok && raw >= a.lo[j] && raw <= a.hi[j];
+        }
+    }
+    // QB * kOut is a multiple of 32: every lane of the warp is here
+    const unsigned votes = __ballot_sync(0xffffffffu, ok) >> (lane & ~3);
+    if (in && a.accept && d == 0) {
+      a.accept[q] = 0;
+      if ((votes & 0xFu) == 0xFu) {
+        const int at = atomicAdd(&count, 1);
+        list[at] = q;
+        hit[at] = 0;
+      }
     }
   }
-  float best = 3.0e38f;
-  for (int t0 = 0; t0 < nt; t0 += kGateTile) {
-    const int cnt = min(kGateTile, nt - t0);
-    __syncthreads();
-    for (int k = threadIdx.x; k < cnt * kIn; k += blockDim.x) tile[k] = Xtrain[(size_t)t0 * kIn + k];
-    __syncthreads();
-    for (int j = 0; j < cnt; j++) {
-      float d2 = 0.0f;
+  if (!a.accept) return;
+  __syncthreads();
+  const int m = count;
+  const int share = m >= 5 ? 1 : m >= 3 ? 2 : m == 2 ? 4 : kWarps;  // warps per query
+  const int groups = kWarps / share, part = warp % share;
+  for (int i = warp / share; i < m; i += groups) {
+    const int q = list[i];
+    float mine = 0.0f;
+    if (lane < kIn) mine = xform(a.x[(size_t)q * kIn + lane], lane, a.xin);
+    float xq[kIn];
+#pragma unroll
+    for (int d = 0; d < kIn; d++) xq[d] = __shfl_sync(0xffffffffu, mine, d);
+    bool found = sqrtf(3.0e38f) <= a.nn_cut;  // a cut beyond any distance
+    for (int t0 = part * 32 * kScan; t0 < a.nt && !found; t0 += share * 32 * kScan) {
+      float best = 3.0e38f;
+      float d2[kScan];
+#pragma unroll
+      for (int j = 0; j < kScan; j++) d2[j] = 0.0f;
 #pragma unroll
       for (int d = 0; d < kIn; d++) {
-        const float e = xq[d] - tile[j * kIn + d];
-        d2 += e * e;
+        const float* col = a.Xt + (size_t)d * a.ldt + t0 + lane;  // ldt: padded to whole groups
+#pragma unroll
+        for (int j = 0; j < kScan; j++) {
+          const float e = xq[d] - __ldg(col + 32 * j);
+          d2[j] += e * e;
+        }
       }
-      best = fminf(best, d2);
+#pragma unroll
+      for (int j = 0; j < kScan; j++)
+        if (t0 + lane + 32 * j < a.nt) best = fminf(best, d2[j]);
+      found = __any_sync(0xffffffffu, sqrtf(best) <= a.nn_cut);
+      if (share > 1 && !found) found = __any_sync(0xffffffffu, *(volatile int*)&hit[i] != 0);
+    }
+    if (found && lane == 0) {
+      hit[i] = 1;
+      a.accept[q] = 1;
     }
   }
-  if (q >= n) return;
-  const float nn = sqrtf(best);
-  nn_dist[q] = nn;
-  bool ok = inbox && nn <= nn_cut;
-#pragma unroll
-  for (int d = 0; d < 2; d++) {
-    const float mu = mean[(size_t)q * kOut + d], s = sd[(size_t)q * kOut + d];
-    ok = ok && isfinite(mu) && s <= (d == 0 ? tau : tau_v) * fabsf(mu);
-  }
-  accept[q] = ok ? 1 : 0;
 }
 
 inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
-cudaError_t launch_prep_inputs(const float* x, int n, const Xform& xf, bf16* X, float* Xf,
+cudaError_t launch_prep_inputs(const float* x, int n, const Xform& xf, bf16* X, float* Xf, int ldx,
                                cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  prep_inputs_kernel<<<blocks(n, 128), 128, 0, s>>>(x, n, xf, X, Xf);
+  prep_inputs_kernel<<<blocks(n, 128), 128, 0, s>>>(x, n, xf, X, Xf, ldx);
   return cudaGetLastError();
 }
 
@@ -720,20 +979,52 @@ cudaError_t launch_advance_step(long long* d_step, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_decode(const float* Y, int n, int members, const Xform& yf, float* mean,
-                          float* sd, cudaStream_t s) {
+cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* p, const bf16* Wb,
+                           const Layout& L, int members, float* Y, unsigned* status,
+                           cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  decode_kernel<<<blocks(n, 128), 128, 0, s>>>(Y, n, members, yf, mean, sd);
+  FwdMaps maps;
+  FwdArgs a;
+  a.x = x;
+  a.n = n;
+  a.H = L.nout[0];
+  a.xf = xf;
+  a.p = p;
+  a.P = L.total;
+  a.Y = Y;
+  a.status = status;
+  for (int l = 0; l <= kHidden; l++) {
+    a.b_off[l] = (int)L.b_off[l];
+    cudaError_t e = make_map(&maps.w[l], Wb + L.w_off[l], L.nin[l], L.nout[l], L.nin[l], L.total,
+                             members, 128);
+    if (e != cudaSuccess) return e;
+  }
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(forward_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)fwd_smem_bytes(256, fwd_ring<256>()));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(forward_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)fwd_smem_bytes(256, fwd_ring<512>()));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const dim3 grid(blocks(n, BM), members);
+  if ((long long)grid.x * grid.y <= 152)  // at most one tile per SM
+    forward_kernel<512><<<grid, 512, fwd_smem_bytes(a.H, fwd_ring<512>()), s>>>(maps, a);
+  else
+    forward_kernel<256><<<grid, 256, fwd_smem_bytes(a.H, fwd_ring<256>()), s>>>(maps, a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gate(const float* x, const float* Xq, int n, const float* Xtrain, int nt,
-                        const float* lo, const float* hi, float nn_cut, const float* mean,
-                        const float* sd, float tau, float tau_v, int* accept, float* nn_dist,
-                        cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  gate_kernel<<<blocks(n, 128), 128, 0, s>>>(x, Xq, n, Xtrain, nt, lo, hi, nn_cut, mean, sd, tau,
-                                             tau_v, accept, nn_dist);
+cudaError_t launch_answer(const GateArgs& a, cudaStream_t s) {
+  if (a.n <= 0) return cudaSuccess;
+  // few queries per block while that still leaves SMs idle (8 per block up to
+  // 4096 queries), so that each query gets as many warps as possible
+  if (a.n <= 4096)
+    answer_kernel<8><<<blocks(a.n, 8), kAnswerThreads, 0, s>>>(a);
+  else
+    answer_kernel<64><<<blocks(a.n, 64), kAnswerThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -61,7 +61,8 @@ struct sg_handle_s {
   // training data
   int n_train = 0;
   bf16* X = nullptr;
-  float *T = nullptr, *Xf = nullptr;
+  float *T = nullptr, *Xt = nullptr;  // Xt: transformed FP32 columns [7][ldt], for the gate
+  int ldt = 0, train_cap = 0;
   // minibatch workspace
   bf16 *Xb = nullptr, *Xbt = nullptr;
   float* Tb = nullptr;
@@ -79,12 +80,13 @@ struct sg_handle_s {
   long long* d_sched = nullptr;  // {first step, steps} of the current sg_train call
   cudaStream_t cap = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  // inference workspace (grown on demand)
+  // inference workspace (grown on demand); the answers of a call are one
+  // block, {status word, mean [n][4], sd [n][4], accept [n]}
   int q_cap = 0;
-  float *q_x = nullptr, *q_xf = nullptr, *q_y = nullptr, *q_mean = nullptr, *q_sd = nullptr,
-        *q_nn = nullptr;
-  bf16 *q_x16 = nullptr, *q_h[2] = {};
-  int* q_acc = nullptr;
+  float *q_x = nullptr, *q_y = nullptr, *q_out = nullptr;
+  bf16* q_x16 = nullptr;
+  // pinned staging of small calls' queries and answers
+  float* h_stage = nullptr;
 
   void* dalloc(size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
@@ -104,6 +106,8 @@ struct sg_handle_s {
       if (free_fn) free_fn(b, ctx); else cudaFree(b);
     }
     blocks.clear();
+    if (h_stage) cudaFreeHost(h_stage);
+    h_stage = nullptr;
   }
 };
 
@@ -132,14 +136,18 @@ GemmArgs gemm_args() {
   return a;
 }
 
-ij_status status_check(sg_handle h) {
-  unsigned st = 0;
-  CUDA_TRY(cudaMemcpyAsync(&st, h->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(cudaStreamSynchronize(h->stream));
+ij_status status_of(unsigned st) {
   if (st & kStatusTimeout)
     return fail(IJ_ERR_TIMEOUT, "a tensor-core completion wait ran out of its iteration limit");
   if (st & kStatusNonFinite) return fail(IJ_ERR_NUMERIC, "non-finite training loss");
   return IJ_OK;
+}
+
+ij_status status_check(sg_handle h) {
+  unsigned st = 0;
+  CUDA_TRY(cudaMemcpyAsync(&st, h->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(cudaStreamSynchronize(h->stream));
+  return status_of(st);
 }
 
 // Forward pass of every member on the minibatch buffers (training layout).
@@ -332,21 +340,21 @@ void fit_xform(const float* a, int n, int dim, int log_mask, Xform& xf) {
   for (int d = dim; d < kInPad; d++) xf.scale[d] = 1.0f;
 }
 
+// Words of the answer block before mean: the status word, padded to 16 bytes.
+constexpr int kOutHead = 4;
+// Calls of up to this many queries go through the pinned staging buffer: one
+// copy in and one copy out (37 KB) instead of one in and four out of pageable
+// memory, each of which the host waits for.
+constexpr int kStagedQueries = 1024;
+
 ij_status ensure_query(sg_handle h, int n) {
   if (n <= h->q_cap) return IJ_OK;
-  const size_t nn = (size_t)n, K = h->K, H = h->H;
+  const size_t nn = (size_t)n, K = h->K;
   h->q_x = (float*)h->dalloc(nn * kIn * 4);
-  h->q_xf = (float*)h->dalloc(nn * kIn * 4);
   h->q_x16 = (bf16*)h->dalloc(nn * kInPad * 2);
-  h->q_h[0] = (bf16*)h->dalloc(K * nn * H * 2);
-  h->q_h[1] = (bf16*)h->dalloc(K * nn * H * 2);
-  h->q_y = (float*)h->dalloc(K * nn * kOutPad * 4);
-  h->q_mean = (float*)h->dalloc(nn * kOut * 4);
-  h->q_sd = (float*)h->dalloc(nn * kOut * 4);
-  h->q_nn = (float*)h->dalloc(nn * 4);
-  h->q_acc = (int*)h->dalloc(nn * 4);
-  if (!h->q_x || !h->q_xf || !h->q_x16 || !h->q_h[0] || !h->q_h[1] || !h->q_y || !h->q_mean ||
-      !h->q_sd || !h->q_nn || !h->q_acc)
+  h->q_y = (float*)h->dalloc(K * nn * kOut * 4);
+  h->q_out = (float*)h->dalloc((kOutHead + nn * (2 * kOut + 1)) * 4);
+  if (!h->q_x || !h->q_x16 || !h->q_y || !h->q_out)
     return fail(IJ_ERR_OOM, "device allocation of the query workspace failed");
   h->q_cap = n;
   return IJ_OK;
@@ -503,19 +511,21 @@ ij_status sg_set_data(sg_handle h, const float* x, const float* y, int n) {
   h->nn_cut = (float)(2.0 * sqrt(nn[(size_t)((n - 1) * 0.95)]));
 
   cudaStream_t s = h->stream;
-  if (n > h->n_train) {
+  if (n > h->train_cap) {
+    h->ldt = (n + 127) / 128 * 128;  // the gate reads whole groups of 128 points
     h->X = (bf16*)h->dalloc((size_t)n * kInPad * 2);
     h->T = (float*)h->dalloc((size_t)n * kOut * 4);
-    h->Xf = (float*)h->dalloc((size_t)n * kIn * 4);
-    if (!h->X || !h->T || !h->Xf) return fail(IJ_ERR_OOM, "device allocation of the data failed");
+    h->Xt = (float*)h->dalloc((size_t)h->ldt * kIn * 4);
+    if (!h->X || !h->T || !h->Xt) return fail(IJ_ERR_OOM, "device allocation of the data failed");
+    h->train_cap = n;
   }
   // raw rows staged in the query workspace
   ij_status st = ensure_query(h, n);
   if (st != IJ_OK) return st;
   CUDA_TRY(cudaMemcpyAsync(h->q_x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(cudaMemcpyAsync(h->q_mean, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, h->X, h->Xf, s));
-  CUDA_TRY(launch_prep_targets(h->q_mean, n, h->xout, h->T, s));
+  CUDA_TRY(cudaMemcpyAsync(h->q_out, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
+  CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, h->X, h->Xt, h->ldt, s));
+  CUDA_TRY(launch_prep_targets(h->q_out, n, h->xout, h->T, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_lo, h->lo, kIn * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_hi, h->hi, kIn * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaStreamSynchronize(s));
@@ -570,55 +580,57 @@ ij_status sg_predict(sg_handle h, const float* x, int n, float* mean, float* sd,
   ij_status st = ensure_query(h, n);
   if (st != IJ_OK) return st;
   cudaStream_t s = h->stream;
+  const size_t nn = (size_t)n;
+  const bool staged = !on_device && n <= kStagedQueries;
+  if (staged && !h->h_stage)
+    CUDA_TRY(cudaMallocHost((void**)&h->h_stage,
+                            (kOutHead + (size_t)kStagedQueries * (2 * kOut + 1)) * 4));
   const float* dx = x;
   if (!on_device) {
-    CUDA_TRY(cudaMemcpyAsync(h->q_x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, s));
+    const float* src = x;
+    if (staged) src = (const float*)memcpy(h->h_stage, x, nn * kIn * 4);
+    CUDA_TRY(cudaMemcpyAsync(h->q_x, src, nn * kIn * 4, cudaMemcpyHostToDevice, s));
     dx = h->q_x;
   }
-  CUDA_TRY(launch_prep_inputs(dx, n, h->xin, h->q_x16, h->q_xf, s));
-  const int H = h->H;
-  const long long P = h->L.total;
-  for (int l = 0; l <= kHidden; l++) {
-    GemmArgs a = gemm_args();
-    a.status = h->d_status;
-    a.B = h->Wb + h->L.w_off[l];
-    a.sB = P;
-    a.ldb = h->L.nin[l];
-    a.bias = h->p + h->L.b_off[l];
-    a.sBias = P;
-    a.M = n;
-    a.N = h->L.nout[l];
-    a.K = h->L.nin[l];
-    if (l == 0) {
-      a.A = h->q_x16;
-      a.lda = kInPad;
-      a.sA = 0;  // one input for every member
-    } else {
-      a.A = h->q_h[(l - 1) & 1];
-      a.lda = H;
-      a.sA = (long long)n * H;
-    }
-    if (l < kHidden) {
-      a.epi = EPI_BIAS_GELU;
-      a.Cb = h->q_h[l & 1];
-      a.ldcb = H;
-      a.sCb = (long long)n * H;
-    } else {
-      a.epi = EPI_BIAS_F32;
-      a.Cf = h->q_y;
-      a.ldcf = kOutPad;
-      a.sCf = (long long)n * kOutPad;
-    }
-    CUDA_TRY(launch_gemm(a, h->K, s));
+  CUDA_TRY(launch_forward(dx, n, h->xin, h->p, h->Wb, h->L, h->K, h->q_y, h->d_status, s));
+  GateArgs a;
+  memset(&a, 0, sizeof(a));
+  a.x = dx;
+  a.Y = h->q_y;
+  a.n = n;
+  a.members = h->K;
+  a.xin = h->xin;
+  a.xout = h->xout;
+  a.Xt = h->Xt;
+  a.nt = h->n_train;
+  a.ldt = h->ldt;
+  a.lo = h->d_lo;
+  a.hi = h->d_hi;
+  a.nn_cut = h->nn_cut;
+  a.tau = h->tau;
+  a.tau_v = h->tau_v;
+  a.mean = h->q_out + kOutHead;
+  a.sd = a.mean + nn * kOut;
+  a.accept = accept ? (int*)(a.sd + nn * kOut) : nullptr;
+  a.status = h->d_status;
+  a.status_out = (unsigned*)h->q_out;
+  CUDA_TRY(launch_answer(a, s));
+  if (staged) {
+    const size_t words = kOutHead + nn * (2 * kOut + (accept ? 1 : 0));
+    CUDA_TRY(cudaMemcpyAsync(h->h_stage, h->q_out, words * 4, cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    const float* o = h->h_stage + kOutHead;
+    if (mean) memcpy(mean, o, nn * kOut * 4);
+    if (sd) memcpy(sd, o + nn * kOut, nn * kOut * 4);
+    if (accept) memcpy(accept, o + 2 * nn * kOut, nn * 4);
+    unsigned word;
+    memcpy(&word, h->h_stage, 4);
+    return status_of(word);
   }
-  CUDA_TRY(launch_decode(h->q_y, n, h->K, h->xout, h->q_mean, h->q_sd, s));
-  if (accept)
-    CUDA_TRY(launch_gate(dx, h->q_xf, n, h->Xf, h->n_train, h->d_lo, h->d_hi, h->nn_cut, h->q_mean,
-                         h->q_sd, h->tau, h->tau_v, h->q_acc, h->q_nn, s));
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (mean) CUDA_TRY(cudaMemcpyAsync(mean, h->q_mean, (size_t)n * kOut * 4, kind, s));
-  if (sd) CUDA_TRY(cudaMemcpyAsync(sd, h->q_sd, (size_t)n * kOut * 4, kind, s));
-  if (accept) CUDA_TRY(cudaMemcpyAsync(accept, h->q_acc, (size_t)n * 4, kind, s));
+  if (mean) CUDA_TRY(cudaMemcpyAsync(mean, a.mean, nn * kOut * 4, kind, s));
+  if (sd) CUDA_TRY(cudaMemcpyAsync(sd, a.sd, nn * kOut * 4, kind, s));
+  if (accept) CUDA_TRY(cudaMemcpyAsync(accept, a.accept, nn * 4, kind, s));
   return status_check(h);
 }
 
@@ -678,11 +690,12 @@ ij_status sg_gradients(sg_handle h, const float* x, const float* y, int n, float
   ij_status st = ensure_query(h, n);
   if (st != IJ_OK) return st;
   bf16* x16 = h->q_x16;
-  float* t = h->q_sd;
+  float* yq = h->q_out;  // raw targets, then the transformed ones
+  float* t = h->q_out + (size_t)n * kOut;
   CUDA_TRY(cudaMemcpyAsync(h->q_x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(cudaMemcpyAsync(h->q_mean, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, x16, nullptr, s));
-  CUDA_TRY(launch_prep_targets(h->q_mean, n, h->xout, t, s));
+  CUDA_TRY(cudaMemcpyAsync(yq, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
+  CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, x16, nullptr, 0, s));
+  CUDA_TRY(launch_prep_targets(yq, n, h->xout, t, s));
   // every member sees the same rows: replicate them into the minibatch layout
   for (int mem = 0; mem < h->K; mem++) {
     CUDA_TRY(cudaMemcpyAsync(h->Xb + (size_t)mem * n * kInPad, x16, (size_t)n * kInPad * 2,
