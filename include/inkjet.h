@@ -218,7 +218,7 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  *                the rows of nozzle-wall strips below the nozzle exit
  *                (costlier per row) and ends with the last eighth of each
  *                lattice's rows, both in chunks a quarter as long;
- *   chunk <= 0 : cost-balanced (the default, 0): with S the number of items
+ *   chunk <= 0 : cost-balanced.  0: with S the number of items
  *                the GPU runs at once, each strip's first rows -- 7/8 of its
  *                cost, wall rows counting 2.2 -- are cut into pieces of
  *                equal cost near one S-th of the total (one wave that ends
@@ -226,6 +226,10 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  *                whole strip in equal pieces, no tail; -2: 3/4 and a tail of
  *                shorter pieces; -3, -4, -5: the whole strip in pieces for 2,
  *                3, 4 full waves.
+ *
+ * An untuned handle takes -1 while its lattices give each item only a few
+ * rows, and beyond that the row chunk (8 .. 56) whose list makes one to three
+ * waves of items.
  *
  * ij_tune      -- set chunk (>= -5) and prefetch (block_size: 32, or <= 0
  *                 for every bucket).  Synchronises.
@@ -239,7 +243,8 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  * 3-D handles have one bucket of 512-thread blocks (one CTA per 28 x 12
  * column tile and z chunk); its one tunable is the z chunk: ij_tune takes
  * chunk >= 1 and prefetch 1 (block_size 512 or <= 0), ij_autotune times
- * chunks of 8 .. 256 planes.  Results do not depend on the chunk.
+ * chunks of 8 .. 256 planes and the untuned choice (the chunk whose busiest
+ * CTA has the fewest planes).  Results do not depend on the chunk.
  */
 ij_status ij_tune(ij_handle h, int block_size, int chunk, int prefetch);
 /* ij_use_graph -- run whole diagnostics periods (diag_every steps, or 16

@@ -441,16 +441,9 @@ void balanced_items(ij_handle h, const Bucket& b, int slots) {
   h->items.insert(h->items.end(), tail.begin(), tail.end());
 }
 
-void build_items(ij_handle h) {
-  std::vector<Bucket> old = h->buckets;
+// The work items of every lattice in h->items, cut as b.chunk asks.
+void list_items(ij_handle h, const Bucket& b) {
   h->items.clear();
-  h->buckets.clear();
-  Bucket b{kStepThreads, 0, 0, 0, 0, step_prefetch_for(kStepThreads)};
-  for (const Bucket& o : old)
-    if (o.nthreads == kStepThreads) {
-      b.chunk = o.chunk;
-      b.prefetch = o.prefetch;
-    }
   if (b.chunk <= 0) {
     balanced_items(h, b, step_slots(b.prefetch, h->fp16, h->odd));
   } else {
@@ -500,6 +493,75 @@ void build_items(ij_handle h) {
       h->items.swap(split);
     }
   }
+}
+
+// The chunk of a handle that is not tuned, from its warp rows (strip rows, a
+// half-warp strip counting half) per work item that the GPU runs at once
+// (152 SMs x 12).  Figures: us a step, in brackets with the 7/8 + tail list
+// (0) that every untuned handle took before.
+//  - Few rows per slot (under 12; 30 with one or two lattices; 50 while
+//    lattices have at most four strips, none of them narrow): equal pieces
+//    making one wave (-1).  What runs together then fits in L2 or lies close
+//    together, and an even end matters more than the order of the items:
+//    200 x 1600 16.8 (22.5), 57 x 98 x 229 40.3 (44.8), 1000 x 3000 70.3
+//    (72.7), 17 x 240 x 812 67.9 (72.6, and 81.9 in 32-row chunks).  At most
+//    four whole strips keep list 0 up to 250 rows per slot: 80 x 100 x 1000
+//    191, 218 in row chunks.
+//  - Beyond, row chunks, neighbouring rows of neighbouring strips together,
+//    whose halo reads meet in L2 and whose DRAM pages are shared: the chunk
+//    that makes about 2300 items, one wave and its short last pieces, up to
+//    40 rows per slot of equal lattices or 20 of uneven ones (8 x 200 x 1600
+//    61.5 (71.6), 10 uneven of 1.3 M cells 39.6 (43.3)), about 5000 items
+//    above, 56 rows and an eighth of the height at most (61 x 184 x 456 133
+//    (144), 20 x 200 x 1600 153 (188), 256 uneven lattices of 34.6 M cells
+//    770 (1090)).
+// Over 44 drawn sets of 0.9 to 28 M cells the choice is within 2 % of the best
+// chunk on the average and 1.12 x faster than list 0 (0.98 x at worst).
+int default_chunk(ij_handle h, Bucket b) {
+  double rows = 0.0, full = 0.0;  // full: a whole warp for every strip
+  int strips = 0, ny = 1;
+  bool equal = true;
+  for (const Inst& I : h->inst) {
+    const int last = I.nx % kStripCols, n = (I.nx + kStripCols - 1) / kStripCols;
+    const bool half = last > 0 && last <= kStripCols / 2 - 2;
+    rows += I.ny * (n - (half ? 0.5 : 0.0));
+    full += (double)I.ny * n;
+    strips = std::max(strips, n);
+    ny = std::max(ny, I.ny);
+    equal = equal && I.nx == h->inst[0].nx && I.ny == h->inst[0].ny;
+  }
+  const double per_slot = rows / std::max(1, step_slots(b.prefetch, h->fp16, h->odd));
+  const bool narrow = full > 1.02 * rows;
+  if (per_slot < 12.0 || (h->n_inst <= 2 && per_slot <= 30.0)) return -1;
+  if (strips <= 4 && !narrow && per_slot <= 250.0) return per_slot <= 50.0 ? -1 : 0;
+  constexpr int kLongest = 56;
+  if (per_slot > 200.0) return kLongest;
+  const int want = per_slot < (equal ? 40.0 : 20.0) ? 2300 : 5000;
+  int best = kLongest, off = 1 << 30;
+  for (int chunk = kLongest; chunk >= 8; chunk -= 4) {
+    if (chunk > std::max(8, ny / 8)) continue;
+    b.chunk = chunk;
+    list_items(h, b);
+    const int d = abs((int)h->items.size() - want);
+    if (d < off) {
+      off = d;
+      best = chunk;
+    }
+  }
+  return best;
+}
+
+void build_items(ij_handle h) {
+  std::vector<Bucket> old = h->buckets;
+  h->buckets.clear();
+  Bucket b{kStepThreads, 0, 0, 0, 0, step_prefetch_for(kStepThreads)};
+  if (old.empty()) b.chunk = default_chunk(h, b);
+  for (const Bucket& o : old)
+    if (o.nthreads == kStepThreads) {
+      b.chunk = o.chunk;
+      b.prefetch = o.prefetch;
+    }
+  list_items(h, b);
   b.count = (int)h->items.size();
   // one block per item: the block scheduler hands new blocks to SMs as
   // they free up (measured faster than blocks of several items, which hold
@@ -676,7 +738,46 @@ ij_status upload_items3(ij_handle h) {
   return IJ_OK;
 }
 
-constexpr int kChunk3Default = 80;  // planes of a 3-D work item before tuning
+// The z chunk of a 3-D handle that is not tuned: the one whose busiest CTA
+// marches over the fewest planes (each item takes its planes and about three
+// more: two re-read at its ends, and the start of its pipeline), weighted by
+// 1 + 0.0006 chunk because longer chunks keep fewer neighbouring tiles in step
+// and so lose halo reads in L2.  Measured (us a step) at the choice, against
+// the 80 planes that every lattice took before: 32 x 32 x 160 45.5 (8 planes)
+// and 235, 64 x 64 x 320 142 (40) and 246, 100 x 80 x 300 226 (64) and 270;
+// 2 x 128 x 128 x 640 keeps 80.
+int default_chunk3(const std::vector<Inst3>& inst, int ctas) {
+  static const int kTry[] = {1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15,  16,  18,
+                             20, 22, 24, 26, 28, 30, 32, 36, 40, 44, 48, 56, 64, 72, 80, 96, 128};
+  int best = 80;
+  double best_cost = 1e300;
+  std::vector<int> load;
+  for (int chunk : kTry) {
+    // items in the order of make_items3, item k on CTA k mod ctas
+    load.assign(std::max(1, ctas), 0);
+    long long k = 0;
+    int zc_max = 0;
+    for (const Inst3& I : inst) zc_max = std::max(zc_max, (I.nz + chunk - 1) / chunk);
+    for (int zc = 0; zc < zc_max; zc++)
+      for (const Inst3& I : inst) {
+        const int z0 = zc * chunk;
+        if (z0 >= I.nz) continue;
+        const int tiles = ((I.nx + kTile3X - 1) / kTile3X) * ((I.ny + kTile3Y - 1) / kTile3Y);
+        const int ch = std::min(chunk, I.nz - z0);
+        const int whole = tiles / (int)load.size();
+        if (whole)
+          for (int& v : load) v += whole * (ch + 3);
+        for (int j = 0; j < tiles % (int)load.size(); j++) load[(k + j) % load.size()] += ch + 3;
+        k += tiles;
+      }
+    const double cost = *std::max_element(load.begin(), load.end()) * (1.0 + 0.0006 * chunk);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = chunk;
+    }
+  }
+  return best;
+}
 
 // Allocate and initialise the lattices of a 3-D handle: per lattice two
 // state buffers (f, g_1..6 in the storage format, g_0 and phi with its
@@ -760,7 +861,7 @@ ij_status create3(ij_handle h) {
   int dev = 0, sms = 1;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  h->buckets.assign(1, Bucket{kStep3Threads, 0, 0, sms, kChunk3Default, 1});
+  h->buckets.assign(1, Bucket{kStep3Threads, 0, 0, sms, default_chunk3(h->inst3, sms), 1});
   ij_status st = upload_items3(h);
   if (st != IJ_OK) return st;
   cudaStream_t s = h->stream;
@@ -1218,7 +1319,11 @@ namespace {
 // read the state at t and write only the other buffer, without diagnostics
 // or ghosts: the state is unchanged).
 ij_status autotune3(ij_handle h, int reps) {
-  static const int kChunks3[] = {8, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96, 128, 160, 256};
+  int sms = 1, dev = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int kChunks3[] = {8,  12, 16, 20,  24,  32,  40, 48,
+                          64, 80, 96, 128, 160, 256, default_chunk3(h->inst3, sms)};
   int max_nz = 1;
   for (const Inst3& I : h->inst3) max_nz = std::max(max_nz, I.nz);
   cudaEvent_t e0, e1;

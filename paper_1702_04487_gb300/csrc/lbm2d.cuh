@@ -56,6 +56,7 @@ struct Item {
   int inst, xs, nout, halo, y0, ch, half, y1;
 };
 
+constexpr int kStripCols = 60;     // written columns of one work item
 constexpr int kStepThreads = 32;  // one warp per block, one work item each
 constexpr int kStepBlocksPerSM = 10;  // resident blocks per SM the registers are sized for
 constexpr int kMaxPrefetch = 4;    // rows staged ahead of use: 1 .. 4

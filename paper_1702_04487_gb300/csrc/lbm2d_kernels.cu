@@ -371,7 +371,6 @@ __device__ __forceinline__ void collide_cell(const float (&fr)[9], const float (
 // of (A, B), which are contiguous and 8-byte aligned when nx is even (ODD
 // instantiation: two 4-byte copies).  FP16 storage: 4-byte half pairs of f
 // and g_1..4, 8-byte FP32 pairs of g_0; every update in FP32.
-constexpr int kStripCols = 60;  // written columns of one work item
 constexpr unsigned kFull = 0xffffffffu;
 
 template <int P, bool H>
