@@ -78,6 +78,18 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return d;
 }
 
+// The same in the 64-byte swizzle layout: rows of 64 bytes (32 values of K),
+// 8-row atoms of 512 bytes; swizzle mode 4.  The copy of 16-byte chunk c of
+// row r lies at chunk c ^ ((r >> 1) & 3).
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
 // Instruction descriptor of kind::f16: FP32 accumulator [4,6) = 1, A and B
 // BF16 [7,10) = [10,13) = 1, both K-major, N >> 3 at [17,23), M >> 4 at
 // [24,29).
@@ -115,6 +127,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
 }
 
+// The same for 8 columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 8; j++) v[j] = __uint_as_float(r[j]);
+}
+
 __device__ __forceinline__ float gelu_f(float x) {
   return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));
 }
@@ -149,6 +173,69 @@ __device__ __forceinline__ void tma_load3(uint32_t dst, const CUtensorMap* map, 
       : "memory");
 }
 
+// Thread 0 of a CTA: the K loop of a 128 x BN tile, loads, MMAs and commits;
+// returns once every MMA is done, or false after a wait that gave up.
+// bars[b]: the load of buffer b landed; bars[kStages + b]: its MMAs done.
+template <int BN>
+__device__ bool gemm_pipeline(uint8_t* smem, uint64_t* bars, const CUtensorMap* tmA,
+                              const CUtensorMap* tmB, int m0, int n0, int za, int zb, int K,
+                              uint32_t tmem) {
+  constexpr int kA = BM * BK * 2;
+  constexpr int kStage = stage_bytes<BN>();
+  constexpr uint32_t kIdesc = idesc_bf16(BM, BN);
+  const int nk = (K + BK - 1) / BK;
+  bool ok = true;
+  // slice kt lives in buffer kt % kStages; its load completes phase
+  // (kt / kStages) & 1 of bars[buffer], its MMAs the same phase of
+  // bars[kStages + buffer]
+  auto load = [&](int kt) {
+    const int b = kt % kStages;
+    const uint32_t ta = smem_u32(smem + b * kStage), tb = ta + kA;
+    mbar_expect_tx(smem_u32(&bars[b]), (uint32_t)kStage);
+    tma_load3(ta, tmA, kt * BK, m0, za, smem_u32(&bars[b]));
+    tma_load3(tb, tmB, kt * BK, n0, zb, smem_u32(&bars[b]));
+  };
+  auto phase = [](int kt) { return (uint32_t)((kt / kStages) & 1); };
+  int loaded = 0;     // slices whose loads were issued
+  int landed = 0;     // slices whose loads were seen complete
+  int committed = 0;  // slices whose MMAs were committed
+  int freed = 0;      // slices whose MMAs were seen complete
+  for (; loaded < nk && loaded < kStages; loaded++) load(loaded);
+  for (int kt = 0; kt < nk; kt++) {
+    const int b = kt % kStages;
+    if (!mbar_wait(smem_u32(&bars[b]), phase(kt))) {
+      ok = false;
+      break;
+    }
+    landed = kt + 1;
+    tc_fence_after();
+    const uint32_t ta = smem_u32(smem + b * kStage), tb = ta + kA;
+#pragma unroll
+    for (int k = 0; k < BK / 16; k++)
+      mma_bf16(tmem, sw128_desc(ta + 32 * k), sw128_desc(tb + 32 * k), kIdesc,
+               (kt > 0 || k > 0) ? 1u : 0u);
+    mma_commit(smem_u32(&bars[kStages + b]));
+    committed = kt + 1;
+    // refill the buffer of the previous slice once its MMAs are done
+    if (kt >= 1 && loaded < nk) {
+      if (!mbar_wait(smem_u32(&bars[kStages + (kt - 1) % kStages]), phase(kt - 1))) {
+        ok = false;
+        break;
+      }
+      freed = kt;
+      load(loaded++);
+    }
+  }
+  // Before the accumulator is read, the tensor memory released or the CTA
+  // exits, every copy issued must have landed and every MMA committed must
+  // be done -- also after a timeout above (these waits are bounded too).
+  for (int kt = landed; kt < loaded; kt++)
+    ok = mbar_wait(smem_u32(&bars[kt % kStages]), phase(kt)) && ok;
+  for (int kt = freed > committed - kStages ? freed : committed - kStages; kt < committed; kt++)
+    ok = mbar_wait(smem_u32(&bars[kStages + kt % kStages]), phase(kt)) && ok;
+  return ok;
+}
+
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -156,18 +243,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  constexpr int kA = BM * BK * 2;
   constexpr int kStage = stage_bytes<BN>();
   constexpr uint32_t kCols = tmem_cols<BN>();
-  constexpr uint32_t kIdesc = idesc_bf16(BM, BN);
-  // bars[b]: the load of buffer b landed; bars[kStages + b]: its MMAs done
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int z = blockIdx.z;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-  const int za = a.sA ? z : 0, zb = a.sB ? z : 0;  // a zero stride shares one operand
 
   if (tid == 0) {
 #pragma unroll
@@ -186,58 +268,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  const int nk = (a.K + BK - 1) / BK;
   bool ok = true;
-  if (tid == 0) {
-    // slice kt lives in buffer kt % kStages; its load completes phase
-    // (kt / kStages) & 1 of bars[buffer], its MMAs the same phase of
-    // bars[kStages + buffer]
-    auto load = [&](int kt) {
-      const int b = kt % kStages;
-      const uint32_t ta = smem_u32(smem + b * kStage), tb = ta + kA;
-      mbar_expect_tx(smem_u32(&bars[b]), (uint32_t)kStage);
-      tma_load3(ta, &tmA, kt * BK, m0, za, smem_u32(&bars[b]));
-      tma_load3(tb, &tmB, kt * BK, n0, zb, smem_u32(&bars[b]));
-    };
-    auto phase = [](int kt) { return (uint32_t)((kt / kStages) & 1); };
-    int loaded = 0;     // slices whose loads were issued
-    int landed = 0;     // slices whose loads were seen complete
-    int committed = 0;  // slices whose MMAs were committed
-    int freed = 0;      // slices whose MMAs were seen complete
-    for (; loaded < nk && loaded < kStages; loaded++) load(loaded);
-    for (int kt = 0; kt < nk; kt++) {
-      const int b = kt % kStages;
-      if (!mbar_wait(smem_u32(&bars[b]), phase(kt))) {
-        ok = false;
-        break;
-      }
-      landed = kt + 1;
-      tc_fence_after();
-      const uint32_t ta = smem_u32(smem + b * kStage), tb = ta + kA;
-#pragma unroll
-      for (int k = 0; k < BK / 16; k++)
-        mma_bf16(tmem, sw128_desc(ta + 32 * k), sw128_desc(tb + 32 * k), kIdesc,
-                 (kt > 0 || k > 0) ? 1u : 0u);
-      mma_commit(smem_u32(&bars[kStages + b]));
-      committed = kt + 1;
-      // refill the buffer of the previous slice once its MMAs are done
-      if (kt >= 1 && loaded < nk) {
-        if (!mbar_wait(smem_u32(&bars[kStages + (kt - 1) % kStages]), phase(kt - 1))) {
-          ok = false;
-          break;
-        }
-        freed = kt;
-        load(loaded++);
-      }
-    }
-    // Before the accumulator is read, the tensor memory released or the CTA
-    // exits, every copy issued must have landed and every MMA committed must
-    // be done -- also after a timeout above (these waits are bounded too).
-    for (int kt = landed; kt < loaded; kt++)
-      ok = mbar_wait(smem_u32(&bars[kt % kStages]), phase(kt)) && ok;
-    for (int kt = freed > committed - kStages ? freed : committed - kStages; kt < committed; kt++)
-      ok = mbar_wait(smem_u32(&bars[kStages + kt % kStages]), phase(kt)) && ok;
-  }
+  if (tid == 0) ok = gemm_pipeline<BN>(smem, bars, &tmA, &tmB, m0, n0, 0, 0, a.K, tmem);
   ok = __syncthreads_and(ok);
   tc_fence_after();
 
@@ -245,13 +277,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Epilogue through shared memory (the operand buffers are free once every
     // MMA is done): each warp takes its 32 rows x 16 columns from tensor
     // memory (lane = row), then works row by row -- half-warps on two rows,
-    // lanes along n -- so that bias, aux and every row-major output are read
-    // and written in contiguous runs; the transposed BF16 copy is written
-    // from the lane = row layout, contiguous along m.
+    // lanes along n -- so that C is written in contiguous runs.
     float* T = reinterpret_cast<float*>(smem) + warp * (32 * 17);
-    const int m = m0 + warp * 32 + lane;
-    const bool mrow = m < a.M;
-    const float* bias = a.bias ? a.bias + z * a.sBias : nullptr;
     const int jj = lane & 15, rh = lane >> 4;
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 16) {
@@ -266,33 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 4
       for (int i = 0; i < 16; i++) {
         const int r = 2 * i + rh, mm = m0 + warp * 32 + r;
-        if (mm >= a.M || n >= a.N) continue;
-        float x = T[r * 17 + jj];
-        if (a.epi == EPI_F32) {
-          a.Cf[z * a.sCf + (size_t)mm * a.ldcf + n] = x;
-          continue;
-        }
-        if (a.epi == EPI_BIAS_F32) {
-          a.Cf[z * a.sCf + (size_t)mm * a.ldcf + n] = x + bias[n];
-          continue;
-        }
-        if (a.epi == EPI_BIAS_GELU) {
-          x += bias[n];
-          if (a.Zout) a.Zout[z * a.sZ + (size_t)mm * a.ldz + n] = x;
-          x = gelu_f(x);
-        } else {  // EPI_GELU_BWD
-          x *= gelu_grad_f(a.aux[z * a.sAux + (size_t)mm * a.ldaux + n]);
-        }
-        const bf16 hb = __float2bfloat16_rn(x);
-        if (a.Cb) a.Cb[z * a.sCb + (size_t)mm * a.ldcb + n] = hb;
-        T[r * 17 + jj] = __bfloat162float(hb);  // for the transposed copy
-      }
-      __syncwarp();
-      if (a.Ct && mrow && (a.epi == EPI_BIAS_GELU || a.epi == EPI_GELU_BWD)) {
-#pragma unroll
-        for (int j = 0; j < 16; j++)
-          if (nb + j < a.N)
-            a.Ct[z * a.sCt + (size_t)(nb + j) * a.ldct + m] = __float2bfloat16_rn(T[lane * 17 + j]);
+        if (mm < a.M && n < a.N) a.C[(size_t)mm * a.ldc + n] = T[r * 17 + jj];
       }
       __syncwarp();  // the next chunk overwrites T
     }
@@ -350,11 +351,11 @@ cudaError_t make_map(CUtensorMap* m, const bf16* base, int K, int rows, int ld,
 }
 
 template <int BN>
-cudaError_t launch_bn(const GemmArgs& a, int members, cudaStream_t s) {
+cudaError_t launch_bn(const GemmArgs& a, cudaStream_t s) {
   const size_t smem = gemm_smem_bytes(BN);
   CUtensorMap ma, mb;
-  cudaError_t e0 = make_map(&ma, a.A, a.K, a.M, a.lda, a.sA, a.sA ? members : 1, BM);
-  if (e0 == cudaSuccess) e0 = make_map(&mb, a.B, a.K, a.N, a.ldb, a.sB, a.sB ? members : 1, BN);
+  cudaError_t e0 = make_map(&ma, a.A, a.K, a.M, a.lda, 0, 1, BM);
+  if (e0 == cudaSuccess) e0 = make_map(&mb, a.B, a.K, a.N, a.ldb, 0, 1, BN);
   if (e0 != cudaSuccess) return e0;
   static bool attr = false;
   if (!attr) {
@@ -363,7 +364,7 @@ cudaError_t launch_bn(const GemmArgs& a, int members, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  dim3 grid((a.M + BM - 1) / BM, (a.N + BN - 1) / BN, members);
+  dim3 grid((a.M + BM - 1) / BM, (a.N + BN - 1) / BN);
   gemm_kernel<BN><<<grid, kThreads, smem, s>>>(ma, mb, a);
   return cudaGetLastError();
 }
@@ -374,18 +375,18 @@ size_t gemm_smem_bytes(int bn) {
   return 1024 + kStages * (size_t)(BM * BK * 2 + bn * BK * 2) + 16 * kStages + 16;
 }
 
-cudaError_t launch_gemm(const GemmArgs& a, int members, cudaStream_t s) {
+cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
   // the narrowest tile that covers N, halved (down to 32 columns) while the
   // grid has fewer than ~2 tiles per SM of a 152-SM part
   int bn = a.N <= 16 ? 16 : a.N <= 32 ? 32 : a.N <= 64 ? 64 : a.N <= 128 ? 128 : 256;
   const long long mt = (a.M + BM - 1) / BM;
-  while (bn > 32 && mt * ((a.N + bn - 1) / bn) * members < 304) bn /= 2;
+  while (bn > 32 && mt * ((a.N + bn - 1) / bn) < 304) bn /= 2;
   switch (bn) {
-    case 16: return launch_bn<16>(a, members, s);
-    case 32: return launch_bn<32>(a, members, s);
-    case 64: return launch_bn<64>(a, members, s);
-    case 128: return launch_bn<128>(a, members, s);
-    default: return launch_bn<256>(a, members, s);
+    case 16: return launch_bn<16>(a, s);
+    case 32: return launch_bn<32>(a, s);
+    case 64: return launch_bn<64>(a, s);
+    case 128: return launch_bn<128>(a, s);
+    default: return launch_bn<256>(a, s);
   }
 }
 
@@ -429,81 +430,6 @@ __global__ void prep_targets_kernel(const float* __restrict__ y, int n, const Xf
   for (int d = 0; d < kOut; d++) T[(size_t)r * kOut + d] = xform(y[(size_t)r * kOut + d], d, yf);
 }
 
-__global__ void gather_kernel(const bf16* __restrict__ X, const float* __restrict__ T, int n,
-                              int bm, unsigned long long seed, const long long* __restrict__ d_step,
-                              bf16* __restrict__ Xb, bf16* __restrict__ Xbt,
-                              float* __restrict__ Tb) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x, mem = blockIdx.y;
-  if (r >= bm) return;
-  const unsigned long long ctr =
-      ((unsigned long long)mem << 56) ^ ((unsigned long long)*d_step << 24) ^ (unsigned)r;
-  const int src = (int)(mix64(seed ^ mix64(ctr)) % (unsigned long long)n);
-  const size_t ob = (size_t)mem * bm;
-#pragma unroll
-  for (int d = 0; d < kInPad; d++) {
-    const bf16 v = X[(size_t)src * kInPad + d];
-    Xb[(ob + r) * kInPad + d] = v;
-    Xbt[(size_t)mem * kInPad * bm + (size_t)d * bm + r] = v;
-  }
-#pragma unroll
-  for (int d = 0; d < kOut; d++) Tb[(ob + r) * kOut + d] = T[(size_t)src * kOut + d];
-}
-
-__global__ void loss_kernel(const float* __restrict__ Y, const float* __restrict__ Tb,
-                            const float* __restrict__ w, int bm, bf16* __restrict__ dY,
-                            bf16* __restrict__ dYt, float* __restrict__ dYft, double* loss,
-                            unsigned* status) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x, mem = blockIdx.y;
-  double acc = 0.0;
-  if (r < bm) {
-    const size_t row = (size_t)mem * bm + r;
-    const float inv = 2.0f / (float)(bm * kOut);
-#pragma unroll
-    for (int d = 0; d < kOutPad; d++) {
-      float g = 0.0f;
-      if (d < kOut) {
-        const float diff = Y[row * kOutPad + d] - Tb[row * kOut + d];
-        acc += (double)w[d] * diff * diff;
-        g = inv * w[d] * diff;
-      }
-      const bf16 gb = __float2bfloat16_rn(g);
-      dY[row * kOutPad + d] = gb;
-      dYt[(size_t)mem * kOutPad * bm + (size_t)d * bm + r] = gb;
-      dYft[(size_t)mem * kOutPad * bm + (size_t)d * bm + r] = g;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(loss + mem, acc / (double)(bm * kOut));
-    if (!isfinite(acc)) atomicOr(status, kStatusNonFinite);
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ float to_f(T v);
-template <>
-__device__ __forceinline__ float to_f<float>(float v) {
-  return v;
-}
-template <>
-__device__ __forceinline__ float to_f<bf16>(bf16 v) {
-  return __bfloat162float(v);
-}
-
-// one warp per (member, row)
-template <typename T>
-__global__ void rowsum_kernel(const T* __restrict__ in, int rows, int cols, int ld, long long sin_,
-                              float* __restrict__ out, long long sout) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int mem = blockIdx.y;
-  if (row >= rows) return;
-  const T* p = in + mem * sin_ + (size_t)row * ld;
-  float acc = 0.0f;
-  for (int c = lane; c < cols; c += 32) acc += to_f<T>(p[c]);
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) out[mem * sout + row] = acc;
-}
-
 // Locate flat parameter index i of a member: layer, and whether a weight
 // (row r, column c) or a bias.
 __device__ __forceinline__ void locate(const Layout& L, long long i, int& l, int& r, int& c,
@@ -524,40 +450,6 @@ __device__ __forceinline__ void locate(const Layout& L, long long i, int& l, int
   }
 }
 
-// d_sched (may be null): {first step, number of steps} of the current
-// training call; lr then decays along a half cosine, lr (1 + cos(pi s / S)) / 2
-// at its step s of S.
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, const Layout L, int members, float lr,
-                            float beta1, float beta2, float eps, const long long* __restrict__ d_step,
-                            const long long* __restrict__ d_sched, bf16* __restrict__ Wb,
-                            bf16* __restrict__ WbT) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= L.total * members) return;
-  if (d_sched && d_sched[1] > 0) {
-    const float frac = (float)(*d_step - d_sched[0]) / (float)d_sched[1];
-    lr *= 0.5f * (1.0f + cospif(fminf(fmaxf(frac, 0.0f), 1.0f)));
-  }
-  const float t = (float)(*d_step + 1);
-  const float bc1 = 1.0f - powf(beta1, t), bc2 = 1.0f - powf(beta2, t);
-  const float gi = g[i];
-  const float mi = beta1 * m[i] + (1.0f - beta1) * gi;
-  const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-  p[i] = pi;
-  const long long mem = i / L.total, k = i % L.total;
-  int l, r, c;
-  bool weight;
-  locate(L, k, l, r, c, weight);
-  if (weight) {
-    const bf16 b = __float2bfloat16_rn(pi);
-    Wb[i] = b;
-    WbT[mem * L.total + L.w_off[l] + (long long)c * L.nout[l] + r] = b;
-  }
-}
-
 __global__ void cast_params_kernel(const float* __restrict__ p, const Layout L, int members,
                                    bf16* __restrict__ Wb, bf16* __restrict__ WbT) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -572,8 +464,6 @@ __global__ void cast_params_kernel(const float* __restrict__ p, const Layout L, 
     WbT[mem * L.total + L.w_off[l] + (long long)c * L.nout[l] + r] = b;
   }
 }
-
-__global__ void advance_step_kernel(long long* d_step) { *d_step += 1; }
 
 // ---------------------------------------------------------------------------
 // Inference: all five layers of a 128-row tile of queries for one member in
@@ -796,6 +686,574 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
   }
 }
 
+// ---------------------------------------------------------------------------
+// The network on a thread-block cluster: a training step's forward pass, loss
+// and back-propagation, or a small inference batch.  A cluster of ceil(H / 32)
+// CTAs takes a 128-row tile of one member; CTA c owns units 32 c .. 32 c + 31
+// of every hidden layer.  Per layer it multiplies the tile's whole activation
+// block (in its shared memory) by its 32 rows of the weights, applies the
+// output pass to 128 x 32 values, and sends the BF16 results, one contiguous
+// 8 KB slice of the next activation block, to every other CTA of the cluster
+// (bulk copies into distributed shared memory, counted on the receiver's
+// barrier).  A CTA's own accumulators stay in tensor memory, so
+// back-propagation finds the pre-activations there; its weight rows, forward
+// and transposed, are fetched ahead of use.  The output layer (16 units) is
+// computed by every CTA for itself, and so is the loss gradient.  What the
+// weight gradients need later goes to global memory transposed: inputs, hidden
+// activations, errors.
+//
+// Two activation blocks and no cluster barrier per layer are enough: a CTA
+// sends slices of layer l + 1 only after it received every slice of layer l,
+// which each sender sent after its own products of layer l - 1, the last to
+// read the block that layer l + 1 is written to.
+//
+// Bound by latency: nine dependent layers.  A launch per layer and pass (14
+// GEMMs and 10 small kernels a step, 7 to 20 us each) took 165 us a step at
+// batch 256, H = 256, five members.  16-byte remote stores by every thread
+// instead of the bulk copies took 2.6 us a layer of this kernel's 5.5.
+constexpr int kUnits = 32;  // hidden units of a CTA
+constexpr int kChainThreads = 512;
+constexpr int kSlice = 128 * kUnits * 2;  // bytes of a CTA's slice of an activation block
+constexpr uint32_t kColY = 128, kColB = 160, kChainCols = 256;  // tensor-memory columns
+
+struct ChainMaps {
+  CUtensorMap w[kHidden + 1];   // W_l: boxes of 64 (K) x 32 units (output layer: 16)
+  CUtensorMap wt[kHidden + 1];  // W_l transposed (l >= 1): boxes of 64 x 32
+};
+struct ChainArgs {
+  int rows, H;
+  // inference: raw queries and their transform, outcomes [m][rows][4]
+  const float* x;
+  Xform xf;
+  float* Y;
+  // training: transformed rows and targets, drawn with replacement by a hash
+  // of (seed, member, step, row), or taken in order (direct)
+  const bf16* X;
+  const float* T;
+  int n, direct;
+  unsigned long long seed;
+  const long long* d_step;
+  const float* w;
+  const float* p;
+  long long P;
+  int b_off[kHidden + 1];
+  bf16* Xt;               // [m][16][rows]
+  bf16* Ht[kHidden];      // [m][H][rows]
+  bf16* dZt[kHidden];     // [m][H][rows]
+  bf16* dYt;              // [m][16][rows]
+  float* dYft;            // [m][16][rows]
+  double* loss;           // [m][4 tiles]: one sum per warp of rows
+  unsigned* status;
+};
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;\n" ::: "memory"); }
+
+int chain_ctas(int H) { return (H + kUnits - 1) / kUnits; }
+size_t chain_smem_bytes(int H) {
+  const size_t slices = (H + BK - 1) / BK;
+  return 2 * (size_t)chain_ctas(H) * kSlice + kSlice + slices * (3 * kUnits * 128 + 16 * 128) +
+         2 * kUnits * 128 + kFwdTail + 1024;  // (blocks may end on half a kilobyte multiple)
+}
+
+template <bool TRAIN>
+__global__ void __launch_bounds__(kChainThreads, 1)
+    chain_kernel(const __grid_constant__ ChainMaps maps, const ChainArgs a) {
+  extern __shared__ __align__(1024) uint8_t fwd_smem[];
+  const int H = a.H, slices = (H + BK - 1) / BK;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t rank, nrank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(nrank));
+  const int tile = blockIdx.x / nrank, m0 = tile * BM, z = blockIdx.y;
+  const int u0 = rank * kUnits, nu = H - u0 < kUnits ? H - u0 : kUnits;
+  // shared memory: two activation blocks, the loss gradient's operand, three
+  // weight slots (W_1..3, then W_3..1 transposed), W_0, W_4 transposed, W_4
+  const uint32_t base = smem_u32(fwd_smem);
+  const uint32_t blk = nrank * kSlice, slot = (uint32_t)slices * kUnits * 128;
+  const uint32_t s_dy = base + 2 * blk, s_w = s_dy + kSlice, s_w0 = s_w + 3 * slot;
+  const uint32_t s_wt4 = s_w0 + kUnits * 128, s_w4 = s_wt4 + kUnits * 128;
+  const uint32_t tail = s_w4 + (uint32_t)slices * 16 * 128;
+  // barriers: W_0; the three slots; W_4 and its transpose; MMAs done; slices
+  // of block 0 and 1 received
+  const uint32_t b_w0 = tail, b_slot = tail + 8, b_w4 = tail + 32, b_mma = tail + 40,
+                 b_in = tail + 48;
+  uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(fwd_smem + (tail - base) + 64);
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < 8; i++) mbar_init(tail + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(kChainCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  cluster_arrive();  // waited for before the first copy into another CTA
+  // rows of units u0 .. of a weight matrix, all of K, into `dst`
+  auto fetch = [&](const CUtensorMap* m, int K, int row, int box, uint32_t dst, uint32_t bar) {
+    for (int s = 0; s * BK < K; s++) tma_load3(dst + s * box * 128, m, s * BK, row, z, bar);
+  };
+  if (tid == 0) {
+    mbar_expect_tx(b_w0, kUnits * 128);
+    fetch(&maps.w[0], kInPad, u0, kUnits, s_w0, b_w0);
+    for (int l = 1; l < kHidden; l++) {
+      mbar_expect_tx(b_slot + 8 * (l - 1), slot);
+      fetch(&maps.w[l], H, u0, kUnits, s_w + (l - 1) * slot, b_slot + 8 * (l - 1));
+    }
+    mbar_expect_tx(b_w4, (uint32_t)slices * 16 * 128 + (TRAIN ? kUnits * 128 : 0));
+    fetch(&maps.w[kHidden], H, 0, 16, s_w4, b_w4);
+    if (TRAIN) fetch(&maps.wt[kHidden], kOutPad, u0, kUnits, s_wt4, b_w4);
+  }
+  // 16 BF16 values of a row as columns 0..15 of an operand slice at `s`
+  auto put_row = [&](uint32_t s, const bf16* v) {
+#pragma unroll
+    for (int c = 0; c < 2; c++)
+      *reinterpret_cast<uint4*>(fwd_smem + (s - base) + tid * 64 + ((c ^ ((tid >> 1) & 3)) << 4)) =
+          reinterpret_cast<const uint4*>(v)[c];
+  };
+  // layer 0's operand (every CTA for itself), BF16, columns 7..15 zero
+  const int row = m0 + (tid & 127);
+  const bool row_in = row < a.rows;
+  float target[kOut] = {0.f, 0.f, 0.f, 0.f};
+  if (tid < BM) {
+    __align__(16) bf16 v[kInPad];
+    if (TRAIN) {
+      uint4 q[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+      if (row_in) {
+        int src = row;
+        if (!a.direct) {
+          const unsigned long long ctr = ((unsigned long long)z << 56) ^
+                                         ((unsigned long long)*a.d_step << 24) ^ (unsigned)row;
+          src = (int)(mix64(a.seed ^ mix64(ctr)) % (unsigned long long)a.n);
+        }
+        q[0] = reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad)[0];
+        q[1] = reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad)[1];
+        const float4 t4 = reinterpret_cast<const float4*>(a.T)[src];
+        target[0] = t4.x;
+        target[1] = t4.y;
+        target[2] = t4.z;
+        target[3] = t4.w;
+      }
+      reinterpret_cast<uint4*>(v)[0] = q[0];
+      reinterpret_cast<uint4*>(v)[1] = q[1];
+      if (rank == 0 && row_in)
+#pragma unroll
+        for (int d = 0; d < kInPad; d++) a.Xt[((size_t)z * kInPad + d) * a.rows + row] = v[d];
+    } else {
+#pragma unroll
+      for (int d = 0; d < kInPad; d++)
+        v[d] = __float2bfloat16_rn(d < kIn && row_in ? xform(a.x[(size_t)row * kIn + d], d, a.xf) : 0.0f);
+    }
+    put_row(base, v);
+  }
+  proxy_fence();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *(volatile uint32_t*)tmem_slot;
+  const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+  const bool rows_in = m0 + (warp & 3) * 32 < a.rows;
+  const int col = (warp >> 2) * 8;  // this warp's 8 of the CTA's units
+  const bool mine = rows_in && col < nu;
+  bool ok = true;
+  uint32_t mma_phase = 0, in_phase = 0;  // in_phase: bit b for block b
+  // D[128 x N] at tensor-memory column dcol = (operand slices at sa, K deep)
+  // times (weight rows at sb, `box` rows a 64-wide slice)^T, once barrier `bar`
+  // says the weights are there; block >= 0: once its slices were received
+  auto multiply = [&](uint32_t sa, int block, uint32_t sb, int box, int K, int N, uint32_t dcol,
+                      uint32_t bar, uint32_t parity) {
+    if (tid == 0) {
+      if (!mbar_wait(bar, parity)) ok = false;
+      if (block >= 0) {
+        if (!mbar_wait(b_in + 8 * block, (in_phase >> block) & 1)) ok = false;
+        in_phase ^= 1u << block;
+      }
+      tc_fence_after();
+      const uint32_t id = idesc_bf16(BM, N);
+      for (int k = 0; k < K / 16; k++)
+        mma_bf16(tmem + dcol, sw64_desc(sa + (k >> 1) * kSlice + 32 * (k & 1)),
+                 sw128_desc(sb + (k >> 2) * box * 128 + 32 * (k & 3)), id, k > 0 ? 1u : 0u);
+      mma_commit(b_mma);
+    }
+    __syncwarp();
+    if (!mbar_wait(b_mma, mma_phase)) ok = false;
+    mma_phase ^= 1;
+    __syncwarp();
+    tc_fence_after();
+  };
+  // this CTA's 8 BF16 values of row `row`, units u0 + col .., into block b
+  auto put = [&](const bf16* o, uint32_t b) {
+    const int r = (warp & 3) * 32 + lane;
+    *reinterpret_cast<uint4*>(fwd_smem + b * blk + rank * kSlice + r * 64 +
+                              (((col / 8) ^ ((r >> 1) & 3)) << 4)) =
+        *reinterpret_cast<const uint4*>(o);
+  };
+  // the CTA's slice of block b to every other CTA of the cluster
+  auto send = [&](uint32_t b) {
+    __syncwarp();
+    proxy_fence();
+    tc_fence_before();
+    __syncthreads();
+    if (tid == 0) {
+      mbar_expect_tx(b_in + 8 * b, (nrank - 1) * kSlice);
+      const uint32_t src = base + b * blk + rank * kSlice;
+      for (uint32_t j = 1; j < nrank; j++) {
+        const uint32_t to = rank + j < nrank ? rank + j : rank + j - nrank;
+        uint32_t dst, bar;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(dst) : "r"(src), "r"(to));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(bar) : "r"(b_in + 8 * b), "r"(to));
+        asm volatile(
+            "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2,"
+            " [%3];\n" ::"r"(dst),
+            "r"(src), "r"((uint32_t)kSlice), "r"(bar)
+            : "memory");
+      }
+    }
+    __syncwarp();
+  };
+  // the same values, transposed, to global memory (lane = row: 64-byte runs)
+  auto keep = [&](const bf16* o, bf16* out) {
+    if (!row_in) return;
+    bf16* dst = out + ((size_t)z * H + u0 + col) * a.rows + row;
+#pragma unroll
+    for (int j = 0; j < 8; j++) dst[(size_t)j * a.rows] = o[j];
+  };
+
+  for (int l = 0; l < kHidden; l++) {
+    if (l == 0)
+      multiply(base, -1, s_w0, kUnits, kInPad, nu, 0, b_w0, 0);
+    else
+      multiply(base + (l & 1) * blk, l & 1, s_w + (l - 1) * slot, kUnits, H, nu, l * kUnits,
+               b_slot + 8 * (l - 1), 0);
+    if (TRAIN && tid == 0 && l >= 1) {
+      // this layer's weights are used: the slot takes W_3 .. W_1 transposed
+      mbar_expect_tx(b_slot + 8 * (l - 1), slot);
+      fetch(&maps.wt[kHidden - l], H, u0, kUnits, s_w + (l - 1) * slot, b_slot + 8 * (l - 1));
+    }
+    __syncwarp();
+    if (l == 0) cluster_wait();  // every CTA of the cluster has started
+    __align__(16) bf16 o[8];
+    if (mine) {
+      const float* bias = a.p + z * a.P + a.b_off[l] + u0 + col;
+      float v[8];
+      tmem_ld8(tmem + lanes + l * kUnits + col, v);
+#pragma unroll
+      for (int j = 0; j < 8; j++) o[j] = __float2bfloat16_rn(gelu_f(v[j] + __ldg(bias + j)));
+      put(o, (l + 1) & 1);
+    }
+    send((l + 1) & 1);
+    if (TRAIN && mine) keep(o, a.Ht[l]);
+  }
+  multiply(base, 0, s_w4, 16, H, 16, kColY, b_w4, 0);
+  if (tid < BM && rows_in) {
+    const float* bias = a.p + z * a.P + a.b_off[kHidden];
+    float v[16];
+    tmem_ld16(tmem + lanes + kColY, v);
+    if (!TRAIN) {
+      if (rank == 0 && row_in)
+        *reinterpret_cast<float4*>(a.Y + ((size_t)z * a.rows + row) * kOut) =
+            make_float4(v[0] + __ldg(bias), v[1] + __ldg(bias + 1), v[2] + __ldg(bias + 2),
+                        v[3] + __ldg(bias + 3));
+    } else {
+      // loss 1 / (4 rows) sum w (y - t)^2 and its gradient
+      double acc = 0.0;
+      const float inv = 2.0f / (float)(a.rows * kOut);
+      __align__(16) bf16 o[kOutPad];
+#pragma unroll
+      for (int d = 0; d < kOutPad; d++) {
+        float g = 0.0f;
+        if (d < kOut && row_in) {
+          const float diff = v[d] + __ldg(bias + d) - target[d];
+          acc += (double)a.w[d] * diff * diff;
+          g = inv * a.w[d] * diff;
+        }
+        o[d] = __float2bfloat16_rn(g);
+        if (rank == 0 && row_in) {
+          const size_t at = ((size_t)z * kOutPad + d) * a.rows + row;
+          a.dYt[at] = o[d];
+          a.dYft[at] = g;
+        }
+      }
+      if (rank == 0) {
+        for (int k = 16; k > 0; k >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, k);
+        if (lane == 0) {
+          a.loss[(size_t)z * 4 * (gridDim.x / nrank) + tile * 4 + warp] =
+              acc / (double)(a.rows * kOut);
+          if (!isfinite(acc)) atomicOr(a.status, kStatusNonFinite);
+        }
+      }
+      put_row(s_dy, o);
+    }
+  } else if (TRAIN && rank == 0 && tid < BM && lane == 0) {
+    a.loss[(size_t)z * 4 * (gridDim.x / nrank) + tile * 4 + warp] = 0.0;
+  }
+  if (TRAIN) {
+    __syncwarp();
+    proxy_fence();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    for (int l = kHidden - 1; l >= 0; l--) {
+      // errors of layer l: (errors of layer l + 1) W_{l+1}, times gelu'(z_l)
+      if (l == kHidden - 1)
+        multiply(s_dy, -1, s_wt4, kUnits, kOutPad, nu, kColB, b_w4, 0);
+      else
+        multiply(base + ((l + 1) & 1) * blk, (l + 1) & 1, s_w + (kHidden - 2 - l) * slot, kUnits, H,
+                 nu, kColB, b_slot + 8 * (kHidden - 2 - l), 1);
+      __align__(16) bf16 o[8];
+      if (mine) {
+        const float* bias = a.p + z * a.P + a.b_off[l] + u0 + col;
+        float v[8], zl[8];
+        tmem_ld8(tmem + lanes + kColB + col, v);
+        tmem_ld8(tmem + lanes + l * kUnits + col, zl);
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+          o[j] = __float2bfloat16_rn(v[j] * gelu_grad_f(zl[j] + __ldg(bias + j)));
+        if (l > 0) put(o, l & 1);
+      }
+      if (l > 0) send(l & 1);
+      if (mine) keep(o, a.dZt[l]);
+    }
+  }
+  if (!ok) atomicOr(a.status, kStatusTimeout);
+  if (tid == 0 && !ok) {
+    // a wait gave up: no copy may land and no MMA run after the CTA ends
+    // (bounded again)
+    mbar_wait(b_w0, 0);
+    for (int i = 0; i < 3; i++) {
+      mbar_wait(b_slot + 8 * i, 0);
+      if (TRAIN) mbar_wait(b_slot + 8 * i, 1);
+    }
+    mbar_wait(b_w4, 0);
+    mbar_wait(b_mma, mma_phase ^ 1);
+  }
+  // no CTA ends while another may still send to it or read from it
+  __syncwarp();
+  tc_fence_before();
+  cluster_arrive();
+  cluster_wait();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                 "r"(kChainCols)
+                 : "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Weight gradients and their Adam update in one launch: a CTA per 128 x 64
+// tile of a layer's weights of one member.  The gradient dW = dZ^T A (A the
+// layer's input; K = the minibatch) is accumulated in tensor memory, and the
+// output pass updates the tile's parameters, moments and BF16 copies at once,
+// so gradients never reach memory.  The bias gradients (row sums of dZ^T) of
+// the tile's rows are shared by the CTAs of a row of tiles and taken by warps
+// 1..7 while thread 0 drives the tensor cores.  The CTA that finishes last
+// advances the step counter.
+//
+// Bound by the parameter traffic, 28 bytes a parameter (29 MB for five members
+// of H = 256), which stays in L2; a gradient GEMM per layer, row sums, Adam
+// with strided writes of the transposed copy and a counter launch took 85 us.
+constexpr int kUpdateThreads = 512;
+constexpr int kUpdateBN = 64;
+
+struct UpdateMaps {
+  CUtensorMap a[kHidden + 1];  // dZ_l^T, boxes of 64 (rows of the minibatch) x 128
+  CUtensorMap b[kHidden + 1];  // input of layer l, transposed, boxes of 64 x 64
+};
+struct UpdateArgs {
+  int rows, grads_only;
+  int first[kHidden + 2];  // first tile of each layer
+  Layout L;
+  float *p, *g, *m, *v;
+  bf16 *Wb, *WbT;
+  const bf16* dZt[kHidden];
+  const float* dYft;
+  float lr, beta1, beta2, eps;
+  long long* d_step;
+  const long long* d_sched;
+  unsigned* counter;
+  unsigned* status;
+};
+
+struct AdamStep {
+  float lr, bc1, bc2;
+};
+
+// One parameter: moments, update; returns the new value.
+__device__ __forceinline__ float adam_update(const UpdateArgs& a, const AdamStep& s, size_t i,
+                                             float gi, float m0, float v0, float p0) {
+  // the rounding of each term is written out, so that results do not hang on
+  // the compiler's choice of which product to fuse
+  const float mi = fmaf(1.0f - a.beta1, gi, __fmul_rn(a.beta1, m0));
+  const float vi = fmaf(__fmul_rn(1.0f - a.beta2, gi), gi, __fmul_rn(a.beta2, v0));
+  a.m[i] = mi;
+  a.v[i] = vi;
+  const float pi = p0 - s.lr * (mi / s.bc1) / (sqrtf(vi / s.bc2) + a.eps);
+  a.p[i] = pi;
+  return pi;
+}
+
+__global__ void __launch_bounds__(kUpdateThreads, 1)
+    update_kernel(const __grid_constant__ UpdateMaps maps, const UpdateArgs a) {
+  extern __shared__ __align__(1024) uint8_t fwd_smem[];
+  constexpr int BN = kUpdateBN;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(fwd_smem + kStages * stage_bytes<BN>());
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int z = blockIdx.y;
+  int l = 0;
+#pragma unroll
+  for (int k = 1; k <= kHidden; k++)
+    if ((int)blockIdx.x >= a.first[k]) l = k;
+  const int nin = a.L.nin[l], nout = a.L.nout[l];
+  const int nt = (nin + BN - 1) / BN, tile = blockIdx.x - a.first[l];
+  const int m0 = tile / nt * BM, jt = tile % nt, n0 = jt * BN;
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < 2 * kStages; i++) mbar_init(smem_u32(&bars[i]), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"((uint32_t)tmem_cols<BN>())
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  AdamStep s{a.lr, 1.0f, 1.0f};
+  if (!a.grads_only) {
+    const long long step = *a.d_step;
+    if (a.d_sched && a.d_sched[1] > 0) {
+      const float frac = (float)(step - a.d_sched[0]) / (float)a.d_sched[1];
+      s.lr *= 0.5f * (1.0f + cospif(fminf(fmaxf(frac, 0.0f), 1.0f)));
+    }
+    const float t = (float)(step + 1);
+    s.bc1 = 1.0f - powf(a.beta1, t);
+    s.bc2 = 1.0f - powf(a.beta2, t);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *(volatile uint32_t*)tmem_slot;
+  const size_t member = (size_t)z * a.L.total;
+  // this warp's 32 rows x 16 columns, taken row by row, half-warps on two rows
+  // (64-byte runs of p, m and v), which are fetched before the gradient is there
+  const int mw = m0 + (warp & 3) * 32, jj = lane & 15, rh = lane >> 4;
+  const int c0 = (warp >> 2) * 16, n = n0 + c0 + jj;  // nin is a multiple of 16
+  const bool mine = mw < nout && n0 + c0 < nin;
+  const size_t at = member + a.L.w_off[l] + (size_t)(mw + rh) * nin + n;
+  float pm[16], pv[16], pp[16];
+  if (mine && !a.grads_only) {
+#pragma unroll
+    for (int i = 0; i < 16; i++)
+      if (mw + 2 * i + rh < nout) {
+        pm[i] = a.m[at + (size_t)(2 * i) * nin];
+        pv[i] = a.v[at + (size_t)(2 * i) * nin];
+        pp[i] = a.p[at + (size_t)(2 * i) * nin];
+      }
+  }
+  bool ok = true;
+  if (tid == 0) {
+    ok = gemm_pipeline<BN>(fwd_smem, bars, &maps.a[l], &maps.b[l], m0, n0, z, z, a.rows, tmem);
+  } else if (warp > 0) {
+    // bias gradients of rows m0 + jt, m0 + jt + nt, ..: four rows of a warp at
+    // a time, lanes along the minibatch; lane j then updates row j of the four
+    const int count = (min(BM, nout - m0) - jt + nt - 1) / nt;
+    const bf16* src = l < kHidden ? a.dZt[l] + (size_t)z * nout * a.rows : nullptr;
+    const float* src32 = a.dYft + (size_t)z * kOutPad * a.rows;
+    for (int i0 = (warp - 1) * 4; i0 < count; i0 += 15 * 4) {
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      auto sum_rows = [&](auto* p) {
+#pragma unroll 4
+        for (int c = lane; c < a.rows; c += 32)
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            const int u = m0 + jt + min(i0 + j, count - 1) * nt;
+            acc[j] += (float)p[(size_t)u * a.rows + c];
+          }
+      };
+      if (src)
+        sum_rows(src);
+      else
+        sum_rows(src32);
+      float mine_acc = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_down_sync(0xffffffffu, acc[j], o);
+        const float t = __shfl_sync(0xffffffffu, acc[j], 0);
+        if (lane == j) mine_acc = t;
+      }
+      if (lane < 4 && i0 + lane < count) {
+        const size_t i = member + a.L.b_off[l] + m0 + jt + (i0 + lane) * nt;
+        if (a.grads_only)
+          a.g[i] = mine_acc;
+        else
+          adam_update(a, s, i, mine_acc, a.m[i], a.v[i], a.p[i]);
+      }
+      __syncwarp();
+    }
+  }
+  ok = __syncthreads_and(ok);
+  tc_fence_after();
+  if (ok) {
+    if (mine) {
+      // through shared memory, as the operand ring is free; the transposed
+      // BF16 copy is written from the lane = row layout
+      float* T = reinterpret_cast<float*>(fwd_smem) + warp * (32 * 17);
+      float v[16];
+      tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+      for (int j = 0; j < 16; j++) T[lane * 17 + j] = v[j];
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 16; i++) {
+        const int r = 2 * i + rh;
+        if (mw + r >= nout) continue;
+        const size_t idx = at + (size_t)(2 * i) * nin;
+        const float x = T[r * 17 + jj];
+        if (a.grads_only) {
+          a.g[idx] = x;
+          continue;
+        }
+        const bf16 b = __float2bfloat16_rn(adam_update(a, s, idx, x, pm[i], pv[i], pp[i]));
+        a.Wb[idx] = b;
+        T[r * 17 + jj] = __bfloat162float(b);
+      }
+      __syncwarp();
+      if (!a.grads_only && mw + lane < nout) {
+        bf16* dst = a.WbT + member + a.L.w_off[l] + (size_t)(n0 + c0) * nout + mw + lane;
+#pragma unroll
+        for (int j = 0; j < 16; j++) dst[(size_t)j * nout] = __float2bfloat16_rn(T[lane * 17 + j]);
+      }
+    }
+  } else if (tid == 0) {
+    atomicOr(a.status, kStatusTimeout);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                 "r"((uint32_t)tmem_cols<BN>())
+                 : "memory");
+  }
+  // every CTA has read the step before it counts itself
+  if (tid == 0 && !a.grads_only) {
+    const unsigned total = gridDim.x * gridDim.y;
+    if (atomicInc(a.counter, total - 1) == total - 1) *a.d_step += 1;
+  }
+}
+
 // Answers of QB queries per block: a thread per (query, outcome) decodes and
 // reduces over the members; the queries that pass the box and spread tests
 // are listed, and warps look for a training point within nn_cut of them, a
@@ -918,44 +1376,6 @@ cudaError_t launch_prep_targets(const float* y, int n, const Xform& yf, float* T
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const bf16* X, const float* T, int n, int bm, int members,
-                          unsigned long long seed, const long long* d_step, bf16* Xb, bf16* Xbt,
-                          float* Tb, cudaStream_t s) {
-  gather_kernel<<<dim3(blocks(bm, 128), members), 128, 0, s>>>(X, T, n, bm, seed, d_step, Xb, Xbt,
-                                                                Tb);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_loss(const float* Y, const float* Tb, const float* w, int bm, int members,
-                        bf16* dY, bf16* dYt, float* dYft, double* loss, unsigned* status,
-                        cudaStream_t s) {
-  loss_kernel<<<dim3(blocks(bm, 128), members), 128, 0, s>>>(Y, Tb, w, bm, dY, dYt, dYft, loss,
-                                                              status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_rowsum_bf16(const bf16* in, int rows, int cols, int ld, long long sin_,
-                               float* out, long long sout, int members, cudaStream_t s) {
-  rowsum_kernel<bf16><<<dim3(blocks(rows, 8), members), 256, 0, s>>>(in, rows, cols, ld, sin_, out,
-                                                                     sout);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_rowsum_f32(const float* in, int rows, int cols, int ld, long long sin_,
-                              float* out, long long sout, int members, cudaStream_t s) {
-  rowsum_kernel<float><<<dim3(blocks(rows, 8), members), 256, 0, s>>>(in, rows, cols, ld, sin_, out,
-                                                                      sout);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adam(float* p, const float* g, float* m, float* v, const Layout& L, int members,
-                        float lr, float beta1, float beta2, float eps, const long long* d_step,
-                        const long long* d_sched, bf16* Wb, bf16* WbT, cudaStream_t s) {
-  adam_kernel<<<blocks(L.total * members, 256), 256, 0, s>>>(p, g, m, v, L, members, lr, beta1,
-                                                              beta2, eps, d_step, d_sched, Wb, WbT);
-  return cudaGetLastError();
-}
-
 __global__ void schedule_begin_kernel(const long long* __restrict__ d_step, long long* d_sched,
                                       long long steps) {
   d_sched[0] = *d_step;
@@ -971,11 +1391,6 @@ cudaError_t launch_schedule_begin(const long long* d_step, long long* d_sched, l
 cudaError_t launch_cast_params(const float* p, const Layout& L, int members, bf16* Wb, bf16* WbT,
                                cudaStream_t s) {
   cast_params_kernel<<<blocks(L.total * members, 256), 256, 0, s>>>(p, L, members, Wb, WbT);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_advance_step(long long* d_step, cudaStream_t s) {
-  advance_step_kernel<<<1, 1, 0, s>>>(d_step);
   return cudaGetLastError();
 }
 
@@ -1016,6 +1431,125 @@ cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* 
     forward_kernel<256><<<grid, 256, fwd_smem_bytes(a.H, fwd_ring<256>()), s>>>(maps, a);
   return cudaGetLastError();
 }
+
+namespace {
+
+template <bool TRAIN>
+cudaError_t launch_chain(const ChainMaps& maps, const ChainArgs& a, int members, cudaStream_t s) {
+  const int ctas = chain_ctas(a.H);
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(chain_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)chain_smem_bytes(256));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks(a.rows, BM) * ctas, members);
+  cfg.blockDim = dim3(kChainThreads);
+  cfg.dynamicSmemBytes = chain_smem_bytes(a.H);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, chain_kernel<TRAIN>, maps, a);
+}
+
+// Tensor maps of the members' weights for chain_kernel.
+cudaError_t chain_maps(ChainMaps* m, const Layout& L, int members, const bf16* Wb, const bf16* WbT) {
+  cudaError_t e = cudaSuccess;
+  for (int l = 0; l <= kHidden && e == cudaSuccess; l++) {
+    e = make_map(&m->w[l], Wb + L.w_off[l], L.nin[l], L.nout[l], L.nin[l], L.total, members,
+                 l == kHidden ? kOutPad : kUnits);
+    if (e == cudaSuccess)
+      e = make_map(&m->wt[l], (WbT ? WbT : Wb) + L.w_off[l], L.nout[l], L.nin[l], L.nout[l], L.total,
+                   members, kUnits);
+  }
+  return e;
+}
+
+}  // namespace
+
+cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s) {
+  const Layout& L = t.L;
+  ChainMaps cm;
+  cudaError_t e = chain_maps(&cm, L, t.members, t.Wb, t.WbT);
+  if (e != cudaSuccess) return e;
+  ChainArgs c = {};
+  c.rows = t.rows;
+  c.H = L.nout[0];
+  c.X = t.X;
+  c.T = t.T;
+  c.n = t.n;
+  c.direct = t.direct;
+  c.seed = t.seed;
+  c.d_step = t.d_step;
+  c.w = t.w;
+  c.p = t.p;
+  c.P = L.total;
+  c.Xt = t.Xt;
+  c.dYt = t.dYt;
+  c.dYft = t.dYft;
+  c.loss = t.loss;
+  c.status = t.status;
+  UpdateMaps um;
+  UpdateArgs u = {};
+  u.rows = t.rows;
+  u.grads_only = t.grads_only;
+  u.L = L;
+  u.p = t.p;
+  u.g = t.g;
+  u.m = t.m;
+  u.v = t.v;
+  u.Wb = t.Wb;
+  u.WbT = t.WbT;
+  u.dYft = t.dYft;
+  u.lr = t.lr;
+  u.beta1 = t.beta1;
+  u.beta2 = t.beta2;
+  u.eps = t.eps;
+  u.d_step = t.d_step;
+  u.d_sched = t.d_sched;
+  u.counter = t.counter;
+  u.status = t.status;
+  const int H = c.H;
+  for (int l = 0; l <= kHidden; l++) {
+    c.b_off[l] = (int)L.b_off[l];
+    if (l < kHidden) {
+      c.Ht[l] = t.Ht[l];
+      c.dZt[l] = t.dZt[l];
+      u.dZt[l] = t.dZt[l];
+    }
+    u.first[l + 1] =
+        u.first[l] + (int)blocks(L.nout[l], BM) * (int)blocks(L.nin[l], kUpdateBN);
+    const bf16* A = l < kHidden ? t.dZt[l] : t.dYt;
+    const bf16* B = l > 0 ? t.Ht[l - 1] : t.Xt;
+    const int na = l < kHidden ? H : kOutPad, nb = l > 0 ? H : kInPad;
+    e = make_map(&um.a[l], A, t.rows, na, t.rows, (long long)na * t.rows, t.members, BM);
+    if (e == cudaSuccess)
+      e = make_map(&um.b[l], B, t.rows, nb, t.rows, (long long)nb * t.rows, t.members, kUpdateBN);
+    if (e != cudaSuccess) return e;
+  }
+  static bool attr = false;
+  const size_t smem = kStages * (size_t)stage_bytes<kUpdateBN>() + kFwdTail;
+  if (!attr) {
+    e = cudaFuncSetAttribute(update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  for (int k = 0; k < t.steps; k++) {
+    e = launch_chain<true>(cm, c, t.members, s);
+    if (e != cudaSuccess) return e;
+    update_kernel<<<dim3(u.first[kHidden + 1], t.members), kUpdateThreads, smem, s>>>(um, u);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+int train_loss_parts(int rows) { return 4 * (int)blocks(rows, BM); }
 
 cudaError_t launch_answer(const GateArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;

@@ -63,23 +63,16 @@ struct sg_handle_s {
   bf16* X = nullptr;
   float *T = nullptr, *Xt = nullptr;  // Xt: transformed FP32 columns [7][ldt], for the gate
   int ldt = 0, train_cap = 0;
-  // minibatch workspace
-  bf16 *Xb = nullptr, *Xbt = nullptr;
-  float* Tb = nullptr;
-  float* Z[kHidden] = {};
-  bf16* Ha[kHidden] = {};
-  bf16* Ht[kHidden] = {};
-  float* Y = nullptr;
-  bf16 *dY = nullptr, *dYt = nullptr;
+  // minibatch workspace (TrainArgs)
+  bf16 *Xt_b = nullptr, *dYt = nullptr;
   float* dYft = nullptr;
-  bf16* dZ[2] = {};
-  bf16* dZt[2] = {};
+  bf16* Ht[kHidden] = {};
+  bf16* dZt[kHidden] = {};
+  unsigned* d_counter = nullptr;
   double* d_loss = nullptr;
   unsigned* d_status = nullptr;
   long long* d_step = nullptr;
   long long* d_sched = nullptr;  // {first step, steps} of the current sg_train call
-  cudaStream_t cap = nullptr;
-  cudaGraphExec_t gexec = nullptr;
   // inference workspace (grown on demand); the answers of a call are one
   // block, {status word, mean [n][4], sd [n][4], accept [n]}
   int q_cap = 0;
@@ -100,8 +93,6 @@ struct sg_handle_s {
   }
   void release() {
     if (stream) cudaStreamSynchronize(stream); else cudaDeviceSynchronize();
-    if (gexec) cudaGraphExecDestroy(gexec);
-    if (cap) cudaStreamDestroy(cap);
     for (void* b : blocks) {
       if (free_fn) free_fn(b, ctx); else cudaFree(b);
     }
@@ -130,12 +121,6 @@ Layout make_layout(int H) {
   return L;
 }
 
-GemmArgs gemm_args() {
-  GemmArgs a;
-  memset(&a, 0, sizeof(a));
-  return a;
-}
-
 ij_status status_of(unsigned st) {
   if (st & kStatusTimeout)
     return fail(IJ_ERR_TIMEOUT, "a tensor-core completion wait ran out of its iteration limit");
@@ -150,174 +135,55 @@ ij_status status_check(sg_handle h) {
   return status_of(st);
 }
 
-// Forward pass of every member on the minibatch buffers (training layout).
-cudaError_t enqueue_forward_train(sg_handle h, int bm, cudaStream_t s) {
-  const int H = h->H, K = h->K;
-  const long long P = h->L.total;
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l <= kHidden && e == cudaSuccess; l++) {
-    GemmArgs a = gemm_args();
-    a.status = h->d_status;
-    a.B = h->Wb + h->L.w_off[l];
-    a.sB = P;
-    a.ldb = h->L.nin[l];
-    a.bias = h->p + h->L.b_off[l];
-    a.sBias = P;
-    a.M = bm;
-    a.N = h->L.nout[l];
-    a.K = h->L.nin[l];
-    if (l == 0) {
-      a.A = h->Xb;
-      a.lda = kInPad;
-      a.sA = (long long)bm * kInPad;
-    } else {
-      a.A = h->Ha[l - 1];
-      a.lda = H;
-      a.sA = (long long)bm * H;
-    }
-    if (l < kHidden) {
-      a.epi = EPI_BIAS_GELU;
-      a.Zout = h->Z[l];
-      a.ldz = H;
-      a.sZ = (long long)bm * H;
-      a.Cb = h->Ha[l];
-      a.ldcb = H;
-      a.sCb = (long long)bm * H;
-      a.Ct = h->Ht[l];
-      a.ldct = bm;
-      a.sCt = (long long)H * bm;
-    } else {
-      a.epi = EPI_BIAS_F32;
-      a.Cf = h->Y;
-      a.ldcf = kOutPad;
-      a.sCf = (long long)bm * kOutPad;
-    }
-    e = launch_gemm(a, K, s);
+// Everything a training step or a gradient pass of `rows` rows needs.
+TrainArgs train_args(sg_handle h, int rows) {
+  TrainArgs t;
+  memset(&t, 0, sizeof(t));
+  t.steps = 1;
+  t.members = h->K;
+  t.rows = rows;
+  t.L = h->L;
+  t.X = h->X;
+  t.T = h->T;
+  t.n = h->n_train;
+  t.seed = h->cfg.seed ^ 0x5EEDull;
+  t.w = h->d_w;
+  t.p = h->p;
+  t.g = h->g;
+  t.m = h->m;
+  t.v = h->v;
+  t.Wb = h->Wb;
+  t.WbT = h->WbT;
+  t.Xt = h->Xt_b;
+  t.dYt = h->dYt;
+  t.dYft = h->dYft;
+  for (int l = 0; l < kHidden; l++) {
+    t.Ht[l] = h->Ht[l];
+    t.dZt[l] = h->dZt[l];
   }
-  return e;
+  t.loss = h->d_loss;
+  t.lr = h->cfg.lr;
+  t.beta1 = h->cfg.beta1;
+  t.beta2 = h->cfg.beta2;
+  t.eps = h->cfg.eps;
+  t.d_step = h->d_step;
+  t.d_sched = h->cfg.lr_cosine ? h->d_sched : nullptr;
+  t.counter = h->d_counter;
+  t.status = h->d_status;
+  return t;
 }
 
-// Loss and backward pass into h->g (all members).
-cudaError_t enqueue_backward(sg_handle h, int bm, cudaStream_t s) {
-  const int H = h->H, K = h->K;
-  const long long P = h->L.total;
-  cudaError_t e = launch_loss(h->Y, h->Tb, h->d_w, bm, K, h->dY, h->dYt, h->dYft, h->d_loss,
-                              h->d_status, s);
-  if (e != cudaSuccess) return e;
-  // output layer: gW5 = dY^T H4, gb5 = column sums of dY
-  {
-    GemmArgs a = gemm_args();
-    a.status = h->d_status;
-    a.epi = EPI_F32;
-    a.A = h->dYt;
-    a.lda = bm;
-    a.sA = (long long)kOutPad * bm;
-    a.B = h->Ht[kHidden - 1];
-    a.ldb = bm;
-    a.sB = (long long)H * bm;
-    a.M = kOutPad;
-    a.N = H;
-    a.K = bm;
-    a.Cf = h->g + h->L.w_off[kHidden];
-    a.ldcf = H;
-    a.sCf = P;
-    if ((e = launch_gemm(a, K, s)) != cudaSuccess) return e;
-    if ((e = launch_rowsum_f32(h->dYft, kOutPad, bm, bm, (long long)kOutPad * bm,
-                               h->g + h->L.b_off[kHidden], P, K, s)) != cudaSuccess)
-      return e;
+// Losses of the members from the parts a pass over `rows` rows left.
+ij_status read_losses(sg_handle h, int rows, double* out) {
+  const int parts = train_loss_parts(rows);
+  std::vector<double> v((size_t)h->K * parts);
+  CUDA_TRY(cudaMemcpyAsync(v.data(), h->d_loss, v.size() * 8, cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(cudaStreamSynchronize(h->stream));
+  for (int m = 0; m < h->K; m++) {
+    out[m] = 0.0;
+    for (int j = 0; j < parts; j++) out[m] += v[(size_t)m * parts + j];
   }
-  // dZ of the last hidden layer: (dY W5) * gelu'(Z4)
-  int cur = 0;
-  {
-    GemmArgs a = gemm_args();
-    a.status = h->d_status;
-    a.epi = EPI_GELU_BWD;
-    a.A = h->dY;
-    a.lda = kOutPad;
-    a.sA = (long long)bm * kOutPad;
-    a.B = h->WbT + h->L.w_off[kHidden];
-    a.ldb = kOutPad;
-    a.sB = P;
-    a.M = bm;
-    a.N = H;
-    a.K = kOutPad;
-    a.aux = h->Z[kHidden - 1];
-    a.ldaux = H;
-    a.sAux = (long long)bm * H;
-    a.Cb = h->dZ[cur];
-    a.ldcb = H;
-    a.sCb = (long long)bm * H;
-    a.Ct = h->dZt[cur];
-    a.ldct = bm;
-    a.sCt = (long long)H * bm;
-    if ((e = launch_gemm(a, K, s)) != cudaSuccess) return e;
-  }
-  for (int l = kHidden - 1; l >= 0; l--) {
-    // weight gradient of layer l: dZ_l^T times the layer's input
-    GemmArgs a = gemm_args();
-    a.status = h->d_status;
-    a.epi = EPI_F32;
-    a.A = h->dZt[cur];
-    a.lda = bm;
-    a.sA = (long long)H * bm;
-    if (l == 0) {
-      a.B = h->Xbt;
-      a.sB = (long long)kInPad * bm;
-    } else {
-      a.B = h->Ht[l - 1];
-      a.sB = (long long)H * bm;
-    }
-    a.ldb = bm;
-    a.M = H;
-    a.N = h->L.nin[l];
-    a.K = bm;
-    a.Cf = h->g + h->L.w_off[l];
-    a.ldcf = h->L.nin[l];
-    a.sCf = P;
-    if ((e = launch_gemm(a, K, s)) != cudaSuccess) return e;
-    if ((e = launch_rowsum_bf16(h->dZt[cur], H, bm, bm, (long long)H * bm, h->g + h->L.b_off[l], P,
-                                K, s)) != cudaSuccess)
-      return e;
-    if (l == 0) break;
-    // dZ_{l-1} = (dZ_l W_l) * gelu'(Z_{l-1})
-    GemmArgs b = gemm_args();
-    b.status = h->d_status;
-    b.epi = EPI_GELU_BWD;
-    b.A = h->dZ[cur];
-    b.lda = H;
-    b.sA = (long long)bm * H;
-    b.B = h->WbT + h->L.w_off[l];
-    b.ldb = H;
-    b.sB = P;
-    b.M = bm;
-    b.N = H;
-    b.K = H;
-    b.aux = h->Z[l - 1];
-    b.ldaux = H;
-    b.sAux = (long long)bm * H;
-    b.Cb = h->dZ[cur ^ 1];
-    b.ldcb = H;
-    b.sCb = (long long)bm * H;
-    b.Ct = h->dZt[cur ^ 1];
-    b.ldct = bm;
-    b.sCt = (long long)H * bm;
-    if ((e = launch_gemm(b, K, s)) != cudaSuccess) return e;
-    cur ^= 1;
-  }
-  return cudaSuccess;
-}
-
-cudaError_t enqueue_train_step(sg_handle h, cudaStream_t s) {
-  cudaError_t e = launch_gather(h->X, h->T, h->n_train, h->bm, h->K, h->cfg.seed ^ 0x5EEDull,
-                                h->d_step, h->Xb, h->Xbt, h->Tb, s);
-  if (e == cudaSuccess) e = enqueue_forward_train(h, h->bm, s);
-  if (e == cudaSuccess) e = enqueue_backward(h, h->bm, s);
-  if (e == cudaSuccess)
-    e = launch_adam(h->p, h->g, h->m, h->v, h->L, h->K, h->cfg.lr, h->cfg.beta1, h->cfg.beta2,
-                    h->cfg.eps, h->d_step, h->cfg.lr_cosine ? h->d_sched : nullptr, h->Wb, h->WbT,
-                    s);
-  if (e == cudaSuccess) e = launch_advance_step(h->d_step, s);
-  return e;
+  return IJ_OK;
 }
 
 // Transform (mean, scale) of each column of a [n][dim] host array.
@@ -402,23 +268,15 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   h->v = (float*)h->dalloc(KP * 4);
   h->Wb = (bf16*)h->dalloc(KP * 2);
   h->WbT = (bf16*)h->dalloc(KP * 2);
-  h->Xb = (bf16*)h->dalloc(K * bm * kInPad * 2);
-  h->Xbt = (bf16*)h->dalloc(K * bm * kInPad * 2);
-  h->Tb = (float*)h->dalloc(K * bm * kOut * 4);
+  h->Xt_b = (bf16*)h->dalloc(K * bm * kInPad * 2);
   for (int l = 0; l < kHidden; l++) {
-    h->Z[l] = (float*)h->dalloc(K * bm * H * 4);
-    h->Ha[l] = (bf16*)h->dalloc(K * bm * H * 2);
     h->Ht[l] = (bf16*)h->dalloc(K * bm * H * 2);
+    h->dZt[l] = (bf16*)h->dalloc(K * bm * H * 2);
   }
-  h->Y = (float*)h->dalloc(K * bm * kOutPad * 4);
-  h->dY = (bf16*)h->dalloc(K * bm * kOutPad * 2);
   h->dYt = (bf16*)h->dalloc(K * bm * kOutPad * 2);
   h->dYft = (float*)h->dalloc(K * bm * kOutPad * 4);
-  for (int j = 0; j < 2; j++) {
-    h->dZ[j] = (bf16*)h->dalloc(K * bm * H * 2);
-    h->dZt[j] = (bf16*)h->dalloc(K * bm * H * 2);
-  }
-  h->d_loss = (double*)h->dalloc(K * 8);
+  h->d_loss = (double*)h->dalloc(K * train_loss_parts(h->bm) * 8);
+  h->d_counter = (unsigned*)h->dalloc(4);
   h->d_status = (unsigned*)h->dalloc(4);
   h->d_step = (long long*)h->dalloc(8);
   h->d_sched = (long long*)h->dalloc(16);
@@ -426,15 +284,12 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   h->d_hi = (float*)h->dalloc(kIn * 4);
   h->d_w = (float*)h->dalloc(kOut * 4);
   for (void* b : {(void*)h->p, (void*)h->g, (void*)h->m, (void*)h->v, (void*)h->Wb, (void*)h->WbT,
-                  (void*)h->Xb, (void*)h->Xbt, (void*)h->Tb, (void*)h->Y, (void*)h->dY,
-                  (void*)h->dYt, (void*)h->dYft, (void*)h->d_loss, (void*)h->d_status,
-                  (void*)h->d_step, (void*)h->d_sched, (void*)h->d_lo, (void*)h->d_hi,
-                  (void*)h->d_w})
+                  (void*)h->Xt_b, (void*)h->dYt, (void*)h->dYft, (void*)h->d_loss,
+                  (void*)h->d_counter, (void*)h->d_status, (void*)h->d_step, (void*)h->d_sched,
+                  (void*)h->d_lo, (void*)h->d_hi, (void*)h->d_w})
     if (!b) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
   for (int l = 0; l < kHidden; l++)
-    if (!h->Z[l] || !h->Ha[l] || !h->Ht[l]) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
-  for (int j = 0; j < 2; j++)
-    if (!h->dZ[j] || !h->dZt[j]) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
+    if (!h->Ht[l] || !h->dZt[l]) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
   // He-uniform initialisation on the host (once), zero biases and padding
   std::vector<float> init(KP, 0.0f);
   for (int mem = 0; mem < h->K; mem++)
@@ -458,6 +313,7 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   CUDA_TRY(cudaMemsetAsync(h->v, 0, KP * 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_status, 0, 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_step, 0, 8, s));
+  CUDA_TRY(cudaMemsetAsync(h->d_counter, 0, 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_sched, 0, 16, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_w, cfg->out_weight, kOut * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(launch_cast_params(h->p, h->L, h->K, h->Wb, h->WbT, s));
@@ -530,10 +386,6 @@ ij_status sg_set_data(sg_handle h, const float* x, const float* y, int n) {
   CUDA_TRY(cudaMemcpyAsync(h->d_hi, h->hi, kIn * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   h->n_train = n;
-  if (h->gexec) {  // the captured step bakes in n_train
-    cudaGraphExecDestroy(h->gexec);
-    h->gexec = nullptr;
-  }
   return IJ_OK;
 }
 
@@ -541,32 +393,21 @@ ij_status sg_train(sg_handle h, int steps, double* loss) {
   if (!h) return fail(IJ_ERR_PARAM, "null handle");
   if (steps < 0) return fail(IJ_ERR_PARAM, "steps < 0");
   if (h->n_train < 2) return fail(IJ_ERR_STATE, "no training data (sg_set_data)");
-  if (!h->gexec) {
-    if (!h->cap) CUDA_TRY(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
-    CUDA_TRY(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaMemsetAsync(h->d_loss, 0, h->K * 8, h->cap);
-    if (e == cudaSuccess) e = enqueue_train_step(h, h->cap);
-    cudaGraph_t gr = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(h->cap, &gr);
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-      if (gr) cudaGraphDestroy(gr);
-      return fail(IJ_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
-    }
-    e = cudaGraphInstantiate(&h->gexec, gr, 0);
-    cudaGraphDestroy(gr);
-    if (e != cudaSuccess) return fail(IJ_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-  }
   if (h->cfg.lr_cosine && steps > 0)
     CUDA_TRY(launch_schedule_begin(h->d_step, h->d_sched, steps, h->stream));
-  for (int i = 0; i < steps; i++) CUDA_TRY(cudaGraphLaunch(h->gexec, h->stream));
+  TrainArgs t = train_args(h, h->bm);
+  t.steps = steps;
+  CUDA_TRY(launch_train_step(t, h->stream));
   ij_status st = status_check(h);
   if (st != IJ_OK) return st;
   if (loss) {
-    std::vector<double> l(h->K);
-    CUDA_TRY(cudaMemcpy(l.data(), h->d_loss, h->K * 8, cudaMemcpyDeviceToHost));
-    double s = 0;
-    for (double v : l) s += v;
-    *loss = steps > 0 ? s / h->K : 0.0;
+    *loss = 0.0;
+    if (steps > 0) {
+      std::vector<double> l(h->K);
+      st = read_losses(h, h->bm, l.data());
+      if (st != IJ_OK) return st;
+      for (double v : l) *loss += v / h->K;
+    }
   }
   return IJ_OK;
 }
@@ -696,26 +537,17 @@ ij_status sg_gradients(sg_handle h, const float* x, const float* y, int n, float
   CUDA_TRY(cudaMemcpyAsync(yq, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, x16, nullptr, 0, s));
   CUDA_TRY(launch_prep_targets(yq, n, h->xout, t, s));
-  // every member sees the same rows: replicate them into the minibatch layout
-  for (int mem = 0; mem < h->K; mem++) {
-    CUDA_TRY(cudaMemcpyAsync(h->Xb + (size_t)mem * n * kInPad, x16, (size_t)n * kInPad * 2,
-                             cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(h->Tb + (size_t)mem * n * kOut, t, (size_t)n * kOut * 4,
-                             cudaMemcpyDeviceToDevice, s));
-  }
-  // transpose of the input rows: one column at a time
-  for (int mem = 0; mem < h->K; mem++)
-    for (int d = 0; d < kInPad; d++)
-      CUDA_TRY(cudaMemcpy2DAsync(h->Xbt + (size_t)mem * kInPad * n + (size_t)d * n, 2, x16 + d,
-                                 kInPad * 2, 2, n, cudaMemcpyDeviceToDevice, s));
-  CUDA_TRY(cudaMemsetAsync(h->d_loss, 0, h->K * 8, s));
-  CUDA_TRY(enqueue_forward_train(h, n, s));
-  CUDA_TRY(enqueue_backward(h, n, s));
+  TrainArgs ta = train_args(h, n);
+  ta.direct = 1;  // every member sees the same rows
+  ta.grads_only = 1;
+  ta.X = x16;
+  ta.T = t;
+  ta.n = n;
+  CUDA_TRY(launch_train_step(ta, s));
   st = status_check(h);
   if (st != IJ_OK) return st;
   CUDA_TRY(cudaMemcpy(grads, h->g, (size_t)h->K * h->L.total * 4, cudaMemcpyDeviceToHost));
-  if (loss) CUDA_TRY(cudaMemcpy(loss, h->d_loss, h->K * 8, cudaMemcpyDeviceToHost));
-  return IJ_OK;
+  return loss ? read_losses(h, n, loss) : IJ_OK;
 }
 
 ij_status sg_destroy(sg_handle h) {
@@ -738,7 +570,8 @@ ij_status sg_gemm_bf16(const void* A, int lda, const void* B, int ldb, int M, in
   unsigned* status = nullptr;
   CUDA_TRY(cudaMallocAsync((void**)&status, sizeof(unsigned), s));
   CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(unsigned), s));
-  GemmArgs a = gemm_args();
+  GemmArgs a;
+  memset(&a, 0, sizeof(a));
   a.A = (const bf16*)A;
   a.B = (const bf16*)B;
   a.lda = lda;
@@ -746,11 +579,10 @@ ij_status sg_gemm_bf16(const void* A, int lda, const void* B, int ldb, int M, in
   a.M = M;
   a.N = N;
   a.K = K;
-  a.epi = EPI_F32;
-  a.Cf = C;
-  a.ldcf = ldc;
+  a.C = C;
+  a.ldc = ldc;
   a.status = status;
-  CUDA_TRY(launch_gemm(a, 1, s));
+  CUDA_TRY(launch_gemm(a, s));
   unsigned st = 0;
   CUDA_TRY(cudaMemcpyAsync(&st, status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaFreeAsync(status, s));
