@@ -62,11 +62,11 @@ struct Layout {
 //  receives its parts.
 //  Adam, bias-corrected, at step *d_step + 1; d_sched (may be null): {first
 //  step, step count} of the current training call, over which lr decays along
-//  a half cosine; then *d_step += 1.  grads_only: the gradients go to g and
+//  a half cosine; *d_step advances by `steps` at the end.  grads_only: the gradients go to g and
 //  nothing is updated.
 //  Wb (layout of p) and WbT (layer-wise transposes): BF16 copies of p.
 //  Xt [members][16][rows], Ht, dZt [members][H][rows], dYt, dYft
-//  [members][16][rows]: workspace.  counter: one zeroed word.
+//  [members][16][rows]: workspace.
 struct TrainArgs {
   int steps, members, rows, grads_only;
   Layout L;
@@ -86,7 +86,6 @@ struct TrainArgs {
   float lr, beta1, beta2, eps;
   long long* d_step;
   const long long* d_sched;
-  unsigned* counter;
   unsigned* status;
 };
 cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s);

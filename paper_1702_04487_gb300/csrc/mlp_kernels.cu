@@ -707,10 +707,13 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
 // which each sender sent after its own products of layer l - 1, the last to
 // read the block that layer l + 1 is written to.
 //
-// Bound by latency: nine dependent layers.  A launch per layer and pass (14
-// GEMMs and 10 small kernels a step, 7 to 20 us each) took 165 us a step at
-// batch 256, H = 256, five members.  16-byte remote stores by every thread
-// instead of the bulk copies took 2.6 us a layer of this kernel's 5.5.
+// Bound by latency: nine dependent layers, of which the exchange of the slices
+// (56 KB into every CTA) and the products take 2.1 us, the GELUs 0.8 us; 29 us
+// at batch 256, H = 256, five members, and a training step 47 us with the
+// gradient kernel.  A launch per layer and pass (14 GEMMs and 10 small kernels,
+// 7 to 20 us each) took 165 us a step.  16-byte remote stores by every thread
+// instead of the bulk copies took 2.6 us a layer more than the copies.  Programmatic
+// dependent launch hides the start of each kernel behind the one before.
 constexpr int kUnits = 32;  // hidden units of a CTA
 constexpr int kChainThreads = 512;
 constexpr int kSlice = 128 * kUnits * 2;  // bytes of a CTA's slice of an activation block
@@ -733,6 +736,7 @@ struct ChainArgs {
   int n, direct;
   unsigned long long seed;
   const long long* d_step;
+  long long step_off;     // this launch is step *d_step + step_off
   const float* w;
   const float* p;
   long long P;
@@ -752,7 +756,19 @@ __device__ __forceinline__ void cluster_arrive() {
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
-__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;\n" ::: "memory"); }
+// This CTA's stores to its shared memory are visible to its tensor cores and
+// bulk copies.
+__device__ __forceinline__ void proxy_fence() {
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+// Programmatic dependent launch: wait until the kernel before this one on the
+// stream has finished and its writes are visible; let the next one start.
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+__device__ __forceinline__ void let_next_start() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
 
 int chain_ctas(int H) { return (H + kUnits - 1) / kUnits; }
 size_t chain_smem_bytes(int H) {
@@ -784,6 +800,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   const uint32_t b_w0 = tail, b_slot = tail + 8, b_w4 = tail + 32, b_mma = tail + 40,
                  b_in = tail + 48;
   uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(fwd_smem + (tail - base) + 64);
+  float* const s_bias = reinterpret_cast<float*>(fwd_smem + (tail - base) + 128);  // [5][32]
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < 8; i++) mbar_init(tail + 8 * i, 1);
@@ -802,17 +819,6 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   auto fetch = [&](const CUtensorMap* m, int K, int row, int box, uint32_t dst, uint32_t bar) {
     for (int s = 0; s * BK < K; s++) tma_load3(dst + s * box * 128, m, s * BK, row, z, bar);
   };
-  if (tid == 0) {
-    mbar_expect_tx(b_w0, kUnits * 128);
-    fetch(&maps.w[0], kInPad, u0, kUnits, s_w0, b_w0);
-    for (int l = 1; l < kHidden; l++) {
-      mbar_expect_tx(b_slot + 8 * (l - 1), slot);
-      fetch(&maps.w[l], H, u0, kUnits, s_w + (l - 1) * slot, b_slot + 8 * (l - 1));
-    }
-    mbar_expect_tx(b_w4, (uint32_t)slices * 16 * 128 + (TRAIN ? kUnits * 128 : 0));
-    fetch(&maps.w[kHidden], H, 0, 16, s_w4, b_w4);
-    if (TRAIN) fetch(&maps.wt[kHidden], kOutPad, u0, kUnits, s_wt4, b_w4);
-  }
   // 16 BF16 values of a row as columns 0..15 of an operand slice at `s`
   auto put_row = [&](uint32_t s, const bf16* v) {
 #pragma unroll
@@ -824,15 +830,16 @@ __global__ void __launch_bounds__(kChainThreads, 1)
   const int row = m0 + (tid & 127);
   const bool row_in = row < a.rows;
   float target[kOut] = {0.f, 0.f, 0.f, 0.f};
+  __align__(16) bf16 v0[kInPad];
   if (tid < BM) {
-    __align__(16) bf16 v[kInPad];
     if (TRAIN) {
       uint4 q[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
       if (row_in) {
         int src = row;
         if (!a.direct) {
           const unsigned long long ctr = ((unsigned long long)z << 56) ^
-                                         ((unsigned long long)*a.d_step << 24) ^ (unsigned)row;
+                                         ((unsigned long long)(*a.d_step + a.step_off) << 24) ^
+                                         (unsigned)row;
           src = (int)(mix64(a.seed ^ mix64(ctr)) % (unsigned long long)a.n);
         }
         q[0] = reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad)[0];
@@ -843,18 +850,41 @@ __global__ void __launch_bounds__(kChainThreads, 1)
         target[2] = t4.z;
         target[3] = t4.w;
       }
-      reinterpret_cast<uint4*>(v)[0] = q[0];
-      reinterpret_cast<uint4*>(v)[1] = q[1];
-      if (rank == 0 && row_in)
-#pragma unroll
-        for (int d = 0; d < kInPad; d++) a.Xt[((size_t)z * kInPad + d) * a.rows + row] = v[d];
+      reinterpret_cast<uint4*>(v0)[0] = q[0];
+      reinterpret_cast<uint4*>(v0)[1] = q[1];
     } else {
 #pragma unroll
       for (int d = 0; d < kInPad; d++)
-        v[d] = __float2bfloat16_rn(d < kIn && row_in ? xform(a.x[(size_t)row * kIn + d], d, a.xf) : 0.0f);
+        v0[d] = __float2bfloat16_rn(d < kIn && row_in ? xform(a.x[(size_t)row * kIn + d], d, a.xf) : 0.0f);
     }
-    put_row(base, v);
+    put_row(base, v0);
   }
+  // Up to here nothing depends on the kernel before (the training rows and
+  // the step are constant during a call).  From here on: its parameters; and
+  // it has finished reading what this one overwrites.
+  if (TRAIN) {
+    wait_for_previous();
+    let_next_start();
+  }
+  if (tid == 0) {
+    mbar_expect_tx(b_w0, kUnits * 128);
+    fetch(&maps.w[0], kInPad, u0, kUnits, s_w0, b_w0);
+    for (int l = 1; l < kHidden; l++) {
+      mbar_expect_tx(b_slot + 8 * (l - 1), slot);
+      fetch(&maps.w[l], H, u0, kUnits, s_w + (l - 1) * slot, b_slot + 8 * (l - 1));
+    }
+    mbar_expect_tx(b_w4, (uint32_t)slices * 16 * 128 + (TRAIN ? kUnits * 128 : 0));
+    fetch(&maps.w[kHidden], H, 0, 16, s_w4, b_w4);
+    if (TRAIN) fetch(&maps.wt[kHidden], kOutPad, u0, kUnits, s_wt4, b_w4);
+  }
+  if (tid < (kHidden + 1) * kUnits) {
+    const int l = tid / kUnits, j = tid % kUnits;
+    const int units = l < kHidden ? nu : kOutPad, first = l < kHidden ? u0 : 0;
+    s_bias[tid] = j < units ? __ldcg(a.p + z * a.P + a.b_off[l] + first + j) : 0.0f;
+  }
+  if (TRAIN && tid < BM && rank == 0 && row_in)
+#pragma unroll
+    for (int d = 0; d < kInPad; d++) a.Xt[((size_t)z * kInPad + d) * a.rows + row] = v0[d];
   proxy_fence();
   tc_fence_before();
   __syncthreads();
@@ -878,10 +908,13 @@ __global__ void __launch_bounds__(kChainThreads, 1)
         in_phase ^= 1u << block;
       }
       tc_fence_after();
+      // descriptors count in 16 bytes: 32 bytes a step of K inside a slice
       const uint32_t id = idesc_bf16(BM, N);
+      const uint64_t da = sw64_desc(sa), db = sw128_desc(sb);
+#pragma unroll 4
       for (int k = 0; k < K / 16; k++)
-        mma_bf16(tmem + dcol, sw64_desc(sa + (k >> 1) * kSlice + 32 * (k & 1)),
-                 sw128_desc(sb + (k >> 2) * box * 128 + 32 * (k & 3)), id, k > 0 ? 1u : 0u);
+        mma_bf16(tmem + dcol, da + (uint32_t)((k >> 1) * (kSlice / 16) + 2 * (k & 1)),
+                 db + (uint32_t)((k >> 2) * (box * 8) + 2 * (k & 3)), id, k > 0 ? 1u : 0u);
       mma_commit(b_mma);
     }
     __syncwarp();
@@ -943,59 +976,66 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     if (l == 0) cluster_wait();  // every CTA of the cluster has started
     __align__(16) bf16 o[8];
     if (mine) {
-      const float* bias = a.p + z * a.P + a.b_off[l] + u0 + col;
       float v[8];
       tmem_ld8(tmem + lanes + l * kUnits + col, v);
 #pragma unroll
-      for (int j = 0; j < 8; j++) o[j] = __float2bfloat16_rn(gelu_f(v[j] + __ldg(bias + j)));
+      for (int j = 0; j < 8; j++)
+        o[j] = __float2bfloat16_rn(gelu_f(v[j] + s_bias[l * kUnits + col + j]));
       put(o, (l + 1) & 1);
     }
     send((l + 1) & 1);
     if (TRAIN && mine) keep(o, a.Ht[l]);
   }
   multiply(base, 0, s_w4, 16, H, 16, kColY, b_w4, 0);
+  float diff[kOut] = {0.f, 0.f, 0.f, 0.f};
+  const float inv = 2.0f / (float)(a.rows * kOut);
   if (tid < BM && rows_in) {
-    const float* bias = a.p + z * a.P + a.b_off[kHidden];
+    const float* bias = s_bias + kHidden * kUnits;
     float v[16];
     tmem_ld16(tmem + lanes + kColY, v);
     if (!TRAIN) {
       if (rank == 0 && row_in)
         *reinterpret_cast<float4*>(a.Y + ((size_t)z * a.rows + row) * kOut) =
-            make_float4(v[0] + __ldg(bias), v[1] + __ldg(bias + 1), v[2] + __ldg(bias + 2),
-                        v[3] + __ldg(bias + 3));
+            make_float4(v[0] + bias[0], v[1] + bias[1], v[2] + bias[2], v[3] + bias[3]);
     } else {
-      // loss 1 / (4 rows) sum w (y - t)^2 and its gradient
-      double acc = 0.0;
-      const float inv = 2.0f / (float)(a.rows * kOut);
+      // gradient of the loss 1 / (4 rows) sum w (y - t)^2
       __align__(16) bf16 o[kOutPad];
 #pragma unroll
       for (int d = 0; d < kOutPad; d++) {
         float g = 0.0f;
         if (d < kOut && row_in) {
-          const float diff = v[d] + __ldg(bias + d) - target[d];
-          acc += (double)a.w[d] * diff * diff;
-          g = inv * a.w[d] * diff;
+          diff[d] = v[d] + bias[d] - target[d];
+          g = inv * a.w[d] * diff[d];
         }
         o[d] = __float2bfloat16_rn(g);
-        if (rank == 0 && row_in) {
-          const size_t at = ((size_t)z * kOutPad + d) * a.rows + row;
-          a.dYt[at] = o[d];
-          a.dYft[at] = g;
-        }
-      }
-      if (rank == 0) {
-        for (int k = 16; k > 0; k >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, k);
-        if (lane == 0) {
-          a.loss[(size_t)z * 4 * (gridDim.x / nrank) + tile * 4 + warp] =
-              acc / (double)(a.rows * kOut);
-          if (!isfinite(acc)) atomicOr(a.status, kStatusNonFinite);
-        }
       }
       put_row(s_dy, o);
     }
-  } else if (TRAIN && rank == 0 && tid < BM && lane == 0) {
-    a.loss[(size_t)z * 4 * (gridDim.x / nrank) + tile * 4 + warp] = 0.0;
   }
+  // The loss and what the output layer's gradients need, by the first CTA
+  // while its slices of the next errors are on their way.
+  auto store_loss = [&]() {
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d < kOutPad; d++) {
+      float g = 0.0f;
+      if (d < kOut && row_in) {
+        acc += (double)a.w[d] * diff[d] * diff[d];
+        g = inv * a.w[d] * diff[d];
+      }
+      if (row_in) {
+        const size_t at = ((size_t)z * kOutPad + d) * a.rows + row;
+        a.dYt[at] = __float2bfloat16_rn(g);
+        a.dYft[at] = g;
+      }
+    }
+    for (int k = 16; k > 0; k >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, k);
+    if (lane == 0) {
+      a.loss[(size_t)z * 4 * (gridDim.x / nrank) + tile * 4 + warp] = acc / (double)(a.rows * kOut);
+      if (!isfinite(acc)) atomicOr(a.status, kStatusNonFinite);
+    }
+    __syncwarp();
+  };
   if (TRAIN) {
     __syncwarp();
     proxy_fence();
@@ -1011,17 +1051,17 @@ __global__ void __launch_bounds__(kChainThreads, 1)
                  nu, kColB, b_slot + 8 * (kHidden - 2 - l), 1);
       __align__(16) bf16 o[8];
       if (mine) {
-        const float* bias = a.p + z * a.P + a.b_off[l] + u0 + col;
         float v[8], zl[8];
         tmem_ld8(tmem + lanes + kColB + col, v);
         tmem_ld8(tmem + lanes + l * kUnits + col, zl);
 #pragma unroll
         for (int j = 0; j < 8; j++)
-          o[j] = __float2bfloat16_rn(v[j] * gelu_grad_f(zl[j] + __ldg(bias + j)));
+          o[j] = __float2bfloat16_rn(v[j] * gelu_grad_f(zl[j] + s_bias[l * kUnits + col + j]));
         if (l > 0) put(o, l & 1);
       }
       if (l > 0) send(l & 1);
       if (mine) keep(o, a.dZt[l]);
+      if (l == kHidden - 1 && rank == 0 && tid < BM) store_loss();
     }
   }
   if (!ok) atomicOr(a.status, kStatusTimeout);
@@ -1056,12 +1096,12 @@ __global__ void __launch_bounds__(kChainThreads, 1)
 // output pass updates the tile's parameters, moments and BF16 copies at once,
 // so gradients never reach memory.  The bias gradients (row sums of dZ^T) of
 // the tile's rows are shared by the CTAs of a row of tiles and taken by warps
-// 1..7 while thread 0 drives the tensor cores.  The CTA that finishes last
-// advances the step counter.
+// 1..15 while thread 0 drives the tensor cores.
 //
 // Bound by the parameter traffic, 28 bytes a parameter (29 MB for five members
-// of H = 256), which stays in L2; a gradient GEMM per layer, row sums, Adam
-// with strided writes of the transposed copy and a counter launch took 85 us.
+// of H = 256), which stays in L2, and by Adam's divisions and roots: 9 us; a
+// gradient GEMM per layer, row sums, Adam with strided writes of the transposed
+// copy and a counter launch took 85 us.
 constexpr int kUpdateThreads = 512;
 constexpr int kUpdateBN = 64;
 
@@ -1078,15 +1118,34 @@ struct UpdateArgs {
   const bf16* dZt[kHidden];
   const float* dYft;
   float lr, beta1, beta2, eps;
-  long long* d_step;
+  const long long* d_step;
+  long long step_off;
   const long long* d_sched;
-  unsigned* counter;
   unsigned* status;
 };
 
+// Loads that bypass L1, which may hold the line of an earlier step.
+__device__ __forceinline__ float ld_l2(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ float ld_l2(const bf16* p) {
+  const unsigned short u = __ldcg(reinterpret_cast<const unsigned short*>(p));
+  return __bfloat162float(__ushort_as_bfloat16(u));
+}
+
 struct AdamStep {
-  float lr, bc1, bc2;
+  float lr, bc1, bc2, y1, y2;  // y: reciprocals of bc1, bc2, rounded to nearest
 };
+
+// a / b rounded to nearest, given y = 1 / b rounded to nearest: the quotient
+// a y corrected once by its exact remainder (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000", 1990, theorem on
+// quotients from a correctly rounded reciprocal).  The remainder is exact
+// while it does not underflow; moments below 1e-30, where it may, are far
+// below eps in Adam's denominator.  The general division takes a range check
+// and a branch each, a fifth of this kernel's instructions.
+__device__ __forceinline__ float quotient(float a, float b, float y) {
+  const float q = __fmul_rn(a, y);
+  return fmaf(fmaf(-q, b, a), y, q);
+}
 
 // One parameter: moments, update; returns the new value.
 __device__ __forceinline__ float adam_update(const UpdateArgs& a, const AdamStep& s, size_t i,
@@ -1097,7 +1156,8 @@ __device__ __forceinline__ float adam_update(const UpdateArgs& a, const AdamStep
   const float vi = fmaf(__fmul_rn(1.0f - a.beta2, gi), gi, __fmul_rn(a.beta2, v0));
   a.m[i] = mi;
   a.v[i] = vi;
-  const float pi = p0 - s.lr * (mi / s.bc1) / (sqrtf(vi / s.bc2) + a.eps);
+  const float pi =
+      p0 - s.lr * quotient(mi, s.bc1, s.y1) / (sqrtf(quotient(vi, s.bc2, s.y2)) + a.eps);
   a.p[i] = pi;
   return pi;
 }
@@ -1130,9 +1190,9 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
-  AdamStep s{a.lr, 1.0f, 1.0f};
+  AdamStep s{a.lr, 1.0f, 1.0f, 1.0f, 1.0f};
   if (!a.grads_only) {
-    const long long step = *a.d_step;
+    const long long step = *a.d_step + a.step_off;
     if (a.d_sched && a.d_sched[1] > 0) {
       const float frac = (float)(step - a.d_sched[0]) / (float)a.d_sched[1];
       s.lr *= 0.5f * (1.0f + cospif(fminf(fmaxf(frac, 0.0f), 1.0f)));
@@ -1140,6 +1200,8 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
     const float t = (float)(step + 1);
     s.bc1 = 1.0f - powf(a.beta1, t);
     s.bc2 = 1.0f - powf(a.beta2, t);
+    s.y1 = __frcp_rn(s.bc1);
+    s.y2 = __frcp_rn(s.bc2);
   }
   tc_fence_before();
   __syncthreads();
@@ -1157,11 +1219,15 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
 #pragma unroll
     for (int i = 0; i < 16; i++)
       if (mw + 2 * i + rh < nout) {
-        pm[i] = a.m[at + (size_t)(2 * i) * nin];
-        pv[i] = a.v[at + (size_t)(2 * i) * nin];
-        pp[i] = a.p[at + (size_t)(2 * i) * nin];
+        pm[i] = __ldcg(a.m + at + (size_t)(2 * i) * nin);
+        pv[i] = __ldcg(a.v + at + (size_t)(2 * i) * nin);
+        pp[i] = __ldcg(a.p + at + (size_t)(2 * i) * nin);
       }
   }
+  // Parameters and moments are the previous step's, finished before the
+  // kernel that this one follows let it start; what follows is that kernel's.
+  wait_for_previous();
+  let_next_start();
   bool ok = true;
   if (tid == 0) {
     ok = gemm_pipeline<BN>(fwd_smem, bars, &maps.a[l], &maps.b[l], m0, n0, z, z, a.rows, tmem);
@@ -1179,7 +1245,7 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
 #pragma unroll
           for (int j = 0; j < 4; j++) {
             const int u = m0 + jt + min(i0 + j, count - 1) * nt;
-            acc[j] += (float)p[(size_t)u * a.rows + c];
+            acc[j] += (float)ld_l2(p + (size_t)u * a.rows + c);
           }
       };
       if (src)
@@ -1198,7 +1264,7 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
         if (a.grads_only)
           a.g[i] = mine_acc;
         else
-          adam_update(a, s, i, mine_acc, a.m[i], a.v[i], a.p[i]);
+          adam_update(a, s, i, mine_acc, __ldcg(a.m + i), __ldcg(a.v + i), __ldcg(a.p + i));
       }
       __syncwarp();
     }
@@ -1247,11 +1313,6 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
                  "r"((uint32_t)tmem_cols<BN>())
                  : "memory");
   }
-  // every CTA has read the step before it counts itself
-  if (tid == 0 && !a.grads_only) {
-    const unsigned total = gridDim.x * gridDim.y;
-    if (atomicInc(a.counter, total - 1) == total - 1) *a.d_step += 1;
-  }
 }
 
 // Answers of QB queries per block: a thread per (query, outcome) decodes and
@@ -1283,9 +1344,10 @@ __global__ void __launch_bounds__(kAnswerThreads) answer_kernel(const GateArgs a
   }
   __syncthreads();
   // decode: the four outcomes of a query on four neighbouring lanes
-  for (int k = tid; k < QB * kOut; k += kAnswerThreads) {
+  constexpr int kDecode = QB * kOut < 32 ? 32 : QB * kOut;  // whole warps
+  for (int k = tid; k < kDecode; k += kAnswerThreads) {
     const int q = q0 + (k >> 2), d = k & 3;
-    const bool in = q < a.n;
+    const bool in = q < a.n && k < QB * kOut;
     bool ok = in;
     if (in) {
       double s = 0.0, s2 = 0.0;
@@ -1308,7 +1370,7 @@ __global__ void __launch_bounds__(kAnswerThreads) answer_kernel(const GateArgs a
           ok = ok && raw >= a.lo[j] && raw <= a.hi[j];
         }
     }
-    // QB * kOut is a multiple of 32: every lane of the warp is here
+    // every lane of the warp is here
     const unsigned votes = __ballot_sync(0xffffffffu, ok) >> (lane & ~3);
     if (in && a.accept && d == 0) {
       a.accept[q] = 0;
@@ -1394,10 +1456,74 @@ cudaError_t launch_cast_params(const float* p, const Layout& L, int members, bf1
   return cudaGetLastError();
 }
 
+namespace {
+
+__global__ void advance_step_kernel(long long* d_step, int by) { *d_step += by; }
+
+template <bool TRAIN>
+cudaError_t launch_chain(const ChainMaps& maps, const ChainArgs& a, int members, cudaStream_t s) {
+  const int ctas = chain_ctas(a.H);
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(chain_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)chain_smem_bytes(256));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks(a.rows, BM) * ctas, members);
+  cfg.blockDim = dim3(kChainThreads);
+  cfg.dynamicSmemBytes = chain_smem_bytes(a.H);
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = TRAIN ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, chain_kernel<TRAIN>, maps, a);
+}
+
+// Tensor maps of the members' weights for chain_kernel.
+cudaError_t chain_maps(ChainMaps* m, const Layout& L, int members, const bf16* Wb, const bf16* WbT) {
+  cudaError_t e = cudaSuccess;
+  for (int l = 0; l <= kHidden && e == cudaSuccess; l++) {
+    e = make_map(&m->w[l], Wb + L.w_off[l], L.nin[l], L.nout[l], L.nin[l], L.total, members,
+                 l == kHidden ? kOutPad : kUnits);
+    if (e == cudaSuccess && WbT)
+      e = make_map(&m->wt[l], WbT + L.w_off[l], L.nout[l], L.nin[l], L.nout[l], L.total, members,
+                   kUnits);
+  }
+  return e;
+}
+
+}  // namespace
+
 cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* p, const bf16* Wb,
                            const Layout& L, int members, float* Y, unsigned* status,
                            cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
+  const dim3 grid(blocks(n, BM), members);
+  if ((long long)grid.x * grid.y * chain_ctas(L.nout[0]) <= 152) {
+    // few tiles: a cluster per tile splits the layers (up to 384 queries of
+    // five members of H = 256; a call of one query 49 us, 74 with a CTA per tile)
+    ChainMaps cm = {};
+    cudaError_t e = chain_maps(&cm, L, members, Wb, nullptr);
+    if (e != cudaSuccess) return e;
+    ChainArgs c = {};
+    c.rows = n;
+    c.H = L.nout[0];
+    c.x = x;
+    c.xf = xf;
+    c.Y = Y;
+    c.p = p;
+    c.P = L.total;
+    for (int l = 0; l <= kHidden; l++) c.b_off[l] = (int)L.b_off[l];
+    c.status = status;
+    return launch_chain<false>(cm, c, members, s);
+  }
   FwdMaps maps;
   FwdArgs a;
   a.x = x;
@@ -1424,54 +1550,12 @@ cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* 
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const dim3 grid(blocks(n, BM), members);
   if ((long long)grid.x * grid.y <= 152)  // at most one tile per SM
     forward_kernel<512><<<grid, 512, fwd_smem_bytes(a.H, fwd_ring<512>()), s>>>(maps, a);
   else
     forward_kernel<256><<<grid, 256, fwd_smem_bytes(a.H, fwd_ring<256>()), s>>>(maps, a);
   return cudaGetLastError();
 }
-
-namespace {
-
-template <bool TRAIN>
-cudaError_t launch_chain(const ChainMaps& maps, const ChainArgs& a, int members, cudaStream_t s) {
-  const int ctas = chain_ctas(a.H);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(chain_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)chain_smem_bytes(256));
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks(a.rows, BM) * ctas, members);
-  cfg.blockDim = dim3(kChainThreads);
-  cfg.dynamicSmemBytes = chain_smem_bytes(a.H);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = ctas;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, chain_kernel<TRAIN>, maps, a);
-}
-
-// Tensor maps of the members' weights for chain_kernel.
-cudaError_t chain_maps(ChainMaps* m, const Layout& L, int members, const bf16* Wb, const bf16* WbT) {
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l <= kHidden && e == cudaSuccess; l++) {
-    e = make_map(&m->w[l], Wb + L.w_off[l], L.nin[l], L.nout[l], L.nin[l], L.total, members,
-                 l == kHidden ? kOutPad : kUnits);
-    if (e == cudaSuccess)
-      e = make_map(&m->wt[l], (WbT ? WbT : Wb) + L.w_off[l], L.nout[l], L.nin[l], L.nout[l], L.total,
-                   members, kUnits);
-  }
-  return e;
-}
-
-}  // namespace
 
 cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s) {
   const Layout& L = t.L;
@@ -1513,7 +1597,6 @@ cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s) {
   u.eps = t.eps;
   u.d_step = t.d_step;
   u.d_sched = t.d_sched;
-  u.counter = t.counter;
   u.status = t.status;
   const int H = c.H;
   for (int l = 0; l <= kHidden; l++) {
@@ -1540,11 +1623,25 @@ cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(u.first[kHidden + 1], t.members);
+  cfg.blockDim = dim3(kUpdateThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   for (int k = 0; k < t.steps; k++) {
+    c.step_off = u.step_off = k;
     e = launch_chain<true>(cm, c, t.members, s);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, update_kernel, um, u);
     if (e != cudaSuccess) return e;
-    update_kernel<<<dim3(u.first[kHidden + 1], t.members), kUpdateThreads, smem, s>>>(um, u);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (!t.grads_only && t.steps > 0) {
+    advance_step_kernel<<<1, 1, 0, s>>>(t.d_step, t.steps);
+    return cudaGetLastError();
   }
   return cudaSuccess;
 }
@@ -1553,9 +1650,12 @@ int train_loss_parts(int rows) { return 4 * (int)blocks(rows, BM); }
 
 cudaError_t launch_answer(const GateArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
-  // few queries per block while that still leaves SMs idle (8 per block up to
-  // 4096 queries), so that each query gets as many warps as possible
-  if (a.n <= 4096)
+  // few queries per block while that still leaves SMs idle (one up to three
+  // blocks per SM, 8 up to 4096 queries), so that each query gets as many
+  // warps as possible
+  if (a.n <= 456)
+    answer_kernel<1><<<a.n, kAnswerThreads, 0, s>>>(a);
+  else if (a.n <= 4096)
     answer_kernel<8><<<blocks(a.n, 8), kAnswerThreads, 0, s>>>(a);
   else
     answer_kernel<64><<<blocks(a.n, 64), kAnswerThreads, 0, s>>>(a);

@@ -68,7 +68,6 @@ struct sg_handle_s {
   float* dYft = nullptr;
   bf16* Ht[kHidden] = {};
   bf16* dZt[kHidden] = {};
-  unsigned* d_counter = nullptr;
   double* d_loss = nullptr;
   unsigned* d_status = nullptr;
   long long* d_step = nullptr;
@@ -168,7 +167,6 @@ TrainArgs train_args(sg_handle h, int rows) {
   t.eps = h->cfg.eps;
   t.d_step = h->d_step;
   t.d_sched = h->cfg.lr_cosine ? h->d_sched : nullptr;
-  t.counter = h->d_counter;
   t.status = h->d_status;
   return t;
 }
@@ -276,7 +274,6 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   h->dYt = (bf16*)h->dalloc(K * bm * kOutPad * 2);
   h->dYft = (float*)h->dalloc(K * bm * kOutPad * 4);
   h->d_loss = (double*)h->dalloc(K * train_loss_parts(h->bm) * 8);
-  h->d_counter = (unsigned*)h->dalloc(4);
   h->d_status = (unsigned*)h->dalloc(4);
   h->d_step = (long long*)h->dalloc(8);
   h->d_sched = (long long*)h->dalloc(16);
@@ -285,7 +282,7 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   h->d_w = (float*)h->dalloc(kOut * 4);
   for (void* b : {(void*)h->p, (void*)h->g, (void*)h->m, (void*)h->v, (void*)h->Wb, (void*)h->WbT,
                   (void*)h->Xt_b, (void*)h->dYt, (void*)h->dYft, (void*)h->d_loss,
-                  (void*)h->d_counter, (void*)h->d_status, (void*)h->d_step, (void*)h->d_sched,
+                  (void*)h->d_status, (void*)h->d_step, (void*)h->d_sched,
                   (void*)h->d_lo, (void*)h->d_hi, (void*)h->d_w})
     if (!b) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
   for (int l = 0; l < kHidden; l++)
@@ -313,7 +310,6 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
   CUDA_TRY(cudaMemsetAsync(h->v, 0, KP * 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_status, 0, 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_step, 0, 8, s));
-  CUDA_TRY(cudaMemsetAsync(h->d_counter, 0, 4, s));
   CUDA_TRY(cudaMemsetAsync(h->d_sched, 0, 16, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_w, cfg->out_weight, kOut * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(launch_cast_params(h->p, h->L, h->K, h->Wb, h->WbT, s));
