@@ -229,7 +229,9 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  *
  * An untuned handle takes -1 while its lattices give each item only a few
  * rows, and beyond that the row chunk (8 .. 56) whose list makes one to three
- * waves of items.
+ * waves of items.  Up to 240000 cells, its steps without diagnostics run a
+ * kernel with a block per 16 x 8 tile of cells instead of the list
+ * (ij_autotune times it as one more candidate, ij_tune turns it off).
  *
  * ij_tune      -- set chunk (>= -5) and prefetch (block_size: 32, or <= 0
  *                 for every bucket).  Synchronises.

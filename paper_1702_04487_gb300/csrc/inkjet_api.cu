@@ -60,6 +60,10 @@ struct Bucket {
   int first, count;  // range in the item array
   int grid;
   int chunk, prefetch;
+  // small lattices: steps without diagnostics run a block per tile of cells
+  // (the tiles, cell_count of them, follow the list's items)
+  bool cells;
+  int cell_count;
 };
 
 }  // namespace
@@ -551,15 +555,41 @@ int default_chunk(ij_handle h, Bucket b) {
   return best;
 }
 
+// Whether the steps of an untuned handle run the kernel of small lattices (a
+// block per tile, 1.4 collisions a cell): up to 240000 cells.  Diagnostics
+// steps keep the strips, whose FP32 row sums the records are made of.
+// Measured us a step, in brackets in strips: 64 x 256 4.2 (10.0), 4 x 100 x 400
+// 12.0 (13.7), 400 x 400 10.5 (13.5), 16 x 64 x 256 15.5 (20.7), but 2 x 301 x
+// 501 19.1 (18.0) and 200 x 1600 18.3 (16.8).
+constexpr long long kCellsMost = 240000;
+bool default_cells(ij_handle h) {
+  long long cells = 0;
+  for (const Inst& I : h->inst) cells += (long long)I.nx * I.ny;
+  return cells <= kCellsMost;
+}
+
+// One step of the bucket's items on stream s at time d_t[0] + t_off.
+cudaError_t launch_bucket(ij_handle h, const Bucket& b, int t_off, bool diag, cudaStream_t s) {
+  if (b.cells && !diag)
+    return launch_cells(h->d_inst, h->inst.data(), h->n_inst, h->d_items + b.first + b.count,
+                        b.cell_count, h->d_t, t_off, h->fp16, s);
+  return launch_step(h->d_inst, h->d_items + b.first, b.count, b.nthreads, b.grid, h->d_t, t_off,
+                     diag, b.prefetch, h->fp16, h->odd, s);
+}
+
 void build_items(ij_handle h) {
   std::vector<Bucket> old = h->buckets;
   h->buckets.clear();
-  Bucket b{kStepThreads, 0, 0, 0, 0, step_prefetch_for(kStepThreads)};
-  if (old.empty()) b.chunk = default_chunk(h, b);
+  Bucket b{kStepThreads, 0, 0, 0, 0, step_prefetch_for(kStepThreads), false, 0};
+  if (old.empty()) {
+    b.chunk = default_chunk(h, b);
+    b.cells = default_cells(h);
+  }
   for (const Bucket& o : old)
     if (o.nthreads == kStepThreads) {
       b.chunk = o.chunk;
       b.prefetch = o.prefetch;
+      b.cells = o.cells;
     }
   list_items(h, b);
   b.count = (int)h->items.size();
@@ -567,6 +597,15 @@ void build_items(ij_handle h) {
   // they free up (measured faster than blocks of several items, which hold
   // their slot until the slowest finishes, and than a persistent grid)
   b.grid = (b.count + kStepThreads / 32 - 1) / (kStepThreads / 32);
+  b.cell_count = 0;
+  if (b.cells)
+    for (int k = 0; k < h->n_inst; k++) {
+      const size_t at = h->items.size();
+      const int n = make_cells(h->inst[k], k, nullptr, 0);
+      h->items.resize(at + n);
+      make_cells(h->inst[k], k, h->items.data() + at, n);
+      b.cell_count += n;
+    }
   h->buckets.push_back(b);
 }
 
@@ -641,8 +680,7 @@ ij_status one_step(ij_handle h) {
       e1 = h->get_event();
       CUDA_TRY(cudaEventRecord(e0, h->stream));
     }
-    CUDA_TRY(launch_step(h->d_inst, h->d_items + b.first, b.count, b.nthreads, b.grid, h->d_t, 0,
-                         diag, b.prefetch, h->fp16, h->odd, h->stream));
+    CUDA_TRY(launch_bucket(h, b, 0, diag, h->stream));
     h->launches++;
     if (h->timing) {
       CUDA_TRY(cudaEventRecord(e1, h->stream));
@@ -685,8 +723,7 @@ ij_status build_graph(ij_handle h) {
       e = enqueue_step3(h, cs, j, diag, &n);
     } else {
       for (const Bucket& b : h->buckets) {
-        e = launch_step(h->d_inst, h->d_items + b.first, b.count, b.nthreads, b.grid, h->d_t, j,
-                        diag, b.prefetch, h->fp16, h->odd, cs);
+        e = launch_bucket(h, b, j, diag, cs);
         n++;
         if (e != cudaSuccess) break;
       }
@@ -861,7 +898,7 @@ ij_status create3(ij_handle h) {
   int dev = 0, sms = 1;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  h->buckets.assign(1, Bucket{kStep3Threads, 0, 0, sms, default_chunk3(h->inst3, sms), 1});
+  h->buckets.assign(1, Bucket{kStep3Threads, 0, 0, sms, default_chunk3(h->inst3, sms), 1, false, 0});
   ij_status st = upload_items3(h);
   if (st != IJ_OK) return st;
   cudaStream_t s = h->stream;
@@ -1304,6 +1341,7 @@ ij_status ij_tune(ij_handle h, int block_size, int chunk, int prefetch) {
     if (block_size <= 0 || b.nthreads == block_size) {
       b.chunk = chunk;
       b.prefetch = prefetch;
+      b.cells = false;
     }
   if (!found) return fail(IJ_ERR_PARAM, "no lattice of the handle runs with %d threads", block_size);
   CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -1389,21 +1427,23 @@ ij_status ij_autotune(ij_handle h, int reps) {
       if (block_size_for(h->inst[k]) == nt) max_ny = std::max(max_ny, h->inst[k].ny);
     float best = 1e30f;
     int best_chunk = h->buckets[bi].chunk, best_pf = h->buckets[bi].prefetch;
-    for (int pf = 1; pf <= kMaxPrefetch; pf++)
+    bool best_cells = false;
+    const bool try_cells = default_cells(h);  // one more candidate: pf 0, no list
+    for (int pf = try_cells ? 0 : 1; pf <= kMaxPrefetch; pf++)
       for (int chunk : kChunks) {
         if (chunk > 2 * max_ny && chunk > 0) continue;
-        h->buckets[bi].chunk = chunk;
-        h->buckets[bi].prefetch = pf;
+        if (pf == 0 && chunk != kChunks[0]) continue;
+        h->buckets[bi].cells = pf == 0;
+        h->buckets[bi].chunk = pf ? chunk : best_chunk;
+        h->buckets[bi].prefetch = pf ? pf : best_pf;
         build_items(h);
         st = upload_items(h);
         if (st != IJ_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
         const Bucket& b = h->buckets[bi];
-        CUDA_TRY(launch_step(h->d_inst, h->d_items + b.first, b.count, nt, b.grid, h->d_t, 0,
-                             false, pf, h->fp16, h->odd, h->stream));  // warm-up
+        CUDA_TRY(launch_bucket(h, b, 0, false, h->stream));  // warm-up
         CUDA_TRY(cudaEventRecord(e0, h->stream));
         for (int r = 0; r < reps; r++)
-          CUDA_TRY(launch_step(h->d_inst, h->d_items + b.first, b.count, nt, b.grid, h->d_t, 0,
-                               false, pf, h->fp16, h->odd, h->stream));
+          CUDA_TRY(launch_bucket(h, b, 0, false, h->stream));
         CUDA_TRY(cudaEventRecord(e1, h->stream));
         CUDA_TRY(cudaEventSynchronize(e1));
         float ms = 0.0f;
@@ -1411,10 +1451,12 @@ ij_status ij_autotune(ij_handle h, int reps) {
         h->launches += reps + 1;
         if (ms < best) {
           best = ms;
-          best_chunk = chunk;
-          best_pf = pf;
+          best_cells = b.cells;
+          best_chunk = b.chunk;
+          best_pf = b.prefetch;
         }
       }
+    h->buckets[bi].cells = best_cells;
     h->buckets[bi].chunk = best_chunk;
     h->buckets[bi].prefetch = best_pf;
   }

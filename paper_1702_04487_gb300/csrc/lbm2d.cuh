@@ -88,6 +88,13 @@ cudaError_t launch_init(const Inst* d_inst, const Inst& h_inst, int index, cudaS
 cudaError_t launch_step(const Inst* d_inst, const Item* d_items, int n_items, int nthreads,
                         int grid, const long long* d_t, int t_off, bool diag, int prefetch,
                         bool h16, bool odd, cudaStream_t s);
+// The same step, without diagnostics, by the kernel of small lattices: a block per 16 x 8 tile of
+// cells (make_cells: xs, nout, y0, ch of an item are the tile); any nx.
+// h_inst: the descriptors on the host (device pointers inside).
+cudaError_t launch_cells(const Inst* d_inst, const Inst* h_inst, int n_inst, const Item* d_items,
+                         int n_items, const long long* d_t, int t_off, bool h16, cudaStream_t s);
+// Tiles of one lattice into out (null: count only); -1 when cap is too small.
+int make_cells(const Inst& I, int k, Item* out, int cap);
 // default number of rows staged ahead of use
 int step_prefetch_for(int nthreads);
 // work items the GPU runs at once: SMs x resident blocks of the step kernel

@@ -241,18 +241,28 @@ struct CollK {
   float phis, inv_phis, A4, kappa, omq, inv_tphi, gamma, inv2q, qmt, nu_air, dnu, n0, Fd;
 };
 
+// New g_i: the part that stays and the part that moves in, one rounding for
+// i = 1..3, the product rounded first for i = 4 (its moved part comes a row
+// later in the strip kernel).  Written out, so that every kernel and every
+// branch gives the same bits.
+__device__ __forceinline__ float stay_and_move(float omq, float g, float moved) {
+  return fmaf(omq, g, moved);
+}
+__device__ __forceinline__ float stay4(float omq, float g) { return __fmul_rn(omq, g); }
+
 // Collision of one fluid cell (Eq. 4-6 for f, Eq. 8-10 for g).
 //  fr: f_i - w_i n0 of the cell; g: g_i; phi = sum g (raw); pC .. pSE: phi
 //  with wetting ghosts of the cell and its 8 neighbours.
 //  Out: fs = post-collision f_i - w_i n0 (i = 0..8); gP[i-1] = q g_i +
-//  Omega_i (the part that moves, i = 1..4); gS[i-1] = (1 - q) g_i (the part
-//  that stays); g0n = g_0 + Omega_0; n, uy, u2 of the cell.
+//  Omega_i (the part that moves, i = 1..4; the part (1 - q) g_i stays, see
+//  stay_and_move); g0n = g_0 + Omega_0; n, uy, u2 of the cell.
+template <bool DIAG>
 __device__ __forceinline__ void collide_cell(const float (&fr)[9], const float (&g)[5], float phi,
                                              float pC, float pE, float pN, float pW, float pS,
                                              float pNE, float pNW, float pSW, float pSE,
                                              bool driven, const CollK& K, float (&fs)[9],
-                                             float (&gP)[4], float (&gS)[4], float& g0n, float& n,
-                                             float& uy, float& u2) {
+                                             float (&gP)[4], float& g0n, float& n, float& uy,
+                                             float& u2) {
   // lap = 6 sum_i w_i (phi_i - phi) from the differences, which are exact
   // where neighbours are close (no cancellation of O(10) terms)
   const float lap = (2.0f / 3.0f) * ((pE - pC) + (pN - pC) + (pW - pC) + (pS - pC)) +
@@ -262,7 +272,10 @@ __device__ __forceinline__ void collide_cell(const float (&fr)[9], const float (
   const float gx = (pE - pW) * (1.0f / 3.0f) + (dA_ - dB_) * (1.0f / 12.0f);
   const float gy = (pN - pS) * (1.0f / 3.0f) + (dA_ + dB_) * (1.0f / 12.0f);
   const float mu = K.A4 * phi * ((phi - K.phis) * (phi + K.phis)) - K.kappa * lap;
-  float C = 0.5f * (phi * K.inv_phis + 1.0f);
+  // phi / phi* is rounded first where the diagnostics use it too (DIAG), else
+  // fused; written out, so that every kernel gives the same bits at a step
+  float C = 0.5f * (DIAG ? __fadd_rn(__fmul_rn(phi, K.inv_phis), 1.0f)
+                         : fmaf(phi, K.inv_phis, 1.0f));
   C = fminf(fmaxf(C, 0.0f), 1.0f);
   const float Fb = driven ? K.Fd * C : 0.0f;
   const float Fx = mu * gx, Fy = mu * gy + Fb;
@@ -329,7 +342,6 @@ __device__ __forceinline__ void collide_cell(const float (&fr)[9], const float (
     const float ge = 0.5f * gmu + pq * cu;
     sum_ge += ge;
     gP[i - 1] = fmaf(K.qmt, g[i], ge * K.inv_tphi);  // q g + (ge - g) / tau_phi
-    gS[i - 1] = K.omq * g[i];
   }
   // rest direction: g0_0 = phi - sum_{i>=1} g0_i (Eq. 10 as a balance, so
   // that sum g0 = phi exactly); with phi - g_0 = sum_{i>=1} g_i the
@@ -676,18 +688,18 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
       // ---- collision of row Rc = R-2 (both columns)
       const int Rc = R - 2;
       const int kA2 = KD(1, 2), kB2 = KD(2, 2);
-      float fsA[9], fsB[9], gPA[4], gPB[4], gSA[4], gSB[4], g0A, g0B;
+      float fsA[9], fsB[9], gPA[4], gPB[4], g0A, g0B, ga[5], gb[5];
       float dg[3] = {0.f, 0.f, 0.f};  // row sums of e, e n, e n u_y
       {
-        float ga[5], gb[5], fa[9], fb[9];
+        float fa[9], fb[9];
         load_g((ku + RG::DG - 2) % RG::DG, ga, gb);
         load_f(fr_, fa, fb);
         const bool drv = geom != GEOM_NOZZLE || (m2 >= 0 && m2 < L);
         float nA, uyA, u2A, nB, uyB, u2B;
-        collide_cell(fa, ga, prA2, peA1, peB1, peA0, peW1, peA2, peB0, peW0, peW2, peB2,
-                     drv && dA, K, fsA, gPA, gSA, g0A, nA, uyA, u2A);
-        collide_cell(fb, gb, prB2, peB1, peE1, peB0, peA1, peB2, peE0, peA0, peA2, peE2,
-                     drv && dB, K, fsB, gPB, gSB, g0B, nB, uyB, u2B);
+        collide_cell<DIAG>(fa, ga, prA2, peA1, peB1, peA0, peW1, peA2, peB0, peW0, peW2, peB2,
+                     drv && dA, K, fsA, gPA, g0A, nA, uyA, u2A);
+        collide_cell<DIAG>(fb, gb, prB2, peB1, peE1, peB0, peA1, peB2, peE0, peA0, peA2, peE2,
+                     drv && dB, K, fsB, gPB, g0B, nB, uyB, u2B);
         // only fluid cells whose results are used raise the flag or count
         const bool cA = vA && kA2 == 0, cB = vB && kB2 == 0;
         if ((cA && !(u2A < 0.09f)) || (cB && !(u2B < 0.09f))) atomicOr(I.status, kStatusNumeric);
@@ -844,11 +856,17 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
           if (kE3 != 0) f6B = fsB[8];
         }
         aA[0] = fsA[0]; aA[1] = f1A; aA[2] = f2A; aA[3] = f3A; aA[4] = f5A; aA[5] = f6A;
-        aA[6] = g0A; aA[7] = gSA[0] + p1A; aA[8] = gSA[1] + p2A; aA[9] = gSA[2] + p3A;
-        aA[10] = gSA[3];
+        aA[6] = g0A;
+        aA[7] = stay_and_move(K.omq, ga[1], p1A);
+        aA[8] = stay_and_move(K.omq, ga[2], p2A);
+        aA[9] = stay_and_move(K.omq, ga[3], p3A);
+        aA[10] = stay4(K.omq, ga[4]);
         aB[0] = fsB[0]; aB[1] = f1B; aB[2] = f2B; aB[3] = f3B; aB[4] = f5B; aB[5] = f6B;
-        aB[6] = g0B; aB[7] = gSB[0] + p1B; aB[8] = gSB[1] + p2B; aB[9] = gSB[2] + p3B;
-        aB[10] = gSB[3];
+        aB[6] = g0B;
+        aB[7] = stay_and_move(K.omq, gb[1], p1B);
+        aB[8] = stay_and_move(K.omq, gb[2], p2B);
+        aB[9] = stay_and_move(K.omq, gb[3], p3B);
+        aB[10] = stay4(K.omq, gb[4]);
         upA[0] = fsA[2]; upA[1] = sh5; upA[2] = fsB[6]; upA[3] = gPA[1];
         upB[0] = fsB[2]; upB[1] = fsA[5]; upB[2] = sh6; upB[3] = gPB[1];
         bbA[0] = fsA[5]; bbA[1] = fsA[6];
@@ -869,6 +887,192 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
         atomicAdd(I.sums + 1, tphi);
         atomicAdd(I.sums + 2, tmom);
       }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The step of small lattices: a block per 16 x 8 tile of cells, a thread per
+// colliding cell.  The strip kernel walks three colliding rows and four rows
+// of phi one after the other for every row it writes; a lattice of a few
+// hundred thousand cells does not fill the GPU with such walks and a step
+// takes their serial chain.  Here every population of the tile and its ring is
+// loaded at once, phi of the tile and three rings goes to shared memory, the
+// ring collides too, and the movers are exchanged through shared memory: three
+// block barriers and one chain of a single collision.  The ring makes it 1.4
+// collisions a cell, so larger lattices keep the strips (launch rule in the
+// host code), and so do steps with diagnostics.  The arithmetic and its order
+// are the strip kernel's: results are equal bit for bit.
+//
+// Bound by latency (launch, one round of loads, one collision): 64 x 256 4.2
+// us a step against 10.0 in strips, 128 x 512 6.0 (12.1), 200 x 800 10.7
+// (13.8), 200 x 1600 18.3 (16.8).
+constexpr int kCellX = 16, kCellY = 8;
+constexpr int kCellRX = kCellX + 6, kCellRY = kCellY + 6;  // phi: three rings
+constexpr int kCellCX = kCellX + 2, kCellCY = kCellY + 2;  // colliding cells
+constexpr int kCellThreads = 192;
+static_assert(kCellCX * kCellCY <= kCellThreads, "a thread per colliding cell");
+
+// ONE: a handle of one lattice, whose descriptor comes with the launch and
+// whose tile follows from the block, two dependent loads less.
+template <bool H, bool ONE>
+__global__ void __launch_bounds__(kCellThreads)
+    cell_kernel(const __grid_constant__ Inst one, const Inst* __restrict__ insts,
+                const Item* __restrict__ items, const long long* __restrict__ d_t, int t_off) {
+  __shared__ float sphi[kCellRY][kCellRX];
+  __shared__ unsigned char skind[kCellRY][kCellRX];
+  __shared__ float mv[12][kCellCY * kCellCX];  // f*_1..8, moving g_1..4
+  __shared__ unsigned flag;
+  Item it;
+  if (ONE) {
+    const int tx = (one.nx + kCellX - 1) / kCellX;
+    it.xs = (int)blockIdx.x % tx * kCellX;
+    it.y0 = (int)blockIdx.x / tx * kCellY;
+    it.nout = min(kCellX, one.nx - it.xs);
+    it.ch = min(kCellY, one.ny - it.y0);
+  } else {
+    it = items[blockIdx.x];
+  }
+  const Inst& I = ONE ? one : insts[it.inst];
+  const int tid = threadIdx.x;
+  if (tid == 0) flag = *(volatile const unsigned*)I.status;
+  const long long t = *d_t + t_off;
+  const int nx = I.nx, N = nx * I.ny, x0 = it.xs, y0 = it.y0, nw = it.nout, nh = it.ch;
+  const float* __restrict__ fin = I.f[t & 1];
+  const float* __restrict__ gin = I.g[t & 1];
+  const __half* __restrict__ fhin = reinterpret_cast<const __half*>(fin);
+  const __half* __restrict__ ghin = reinterpret_cast<const __half*>(gin + N);
+  auto load_g = [&](int c, float (&g)[5]) {
+    g[0] = gin[c];
+#pragma unroll
+    for (int i = 1; i < 5; i++)
+      g[i] = H ? __half2float(ghin[(size_t)(i - 1) * N + c]) : gin[(size_t)i * N + c];
+  };
+  // this thread's colliding cell
+  const int cx = tid % kCellCX, cy = tid / kCellCX;
+  const bool coll = cy < nh + 2 && cx < nw + 2;
+  const int x = wrapi(x0 - 1 + cx, nx);
+  int m = 0;
+  const bool mapped = map_row(I, y0 - 1 + cy, m);
+  float fr[9], g[5];
+#pragma unroll
+  for (int i = 0; i < 9; i++) fr[i] = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 5; i++) g[i] = 0.0f;
+  if (coll && mapped) {
+    const int c = m * nx + x;
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+      fr[i] = H ? __half2float(fhin[(size_t)i * N + c]) : fin[(size_t)i * N + c];
+    load_g(c, g);
+  }
+  bool solid = false;
+  for (int k = tid; k < kCellRX * kCellRY; k += kCellThreads) {
+    const int ix = k % kCellRX, iy = k / kCellRX;
+    int kind = 1, mm;
+    float phi = 0.0f;
+    if (ix < nw + 6 && iy < nh + 6) {
+      const int xx = wrapi(x0 - 3 + ix, nx);
+      if (map_row(I, y0 - 3 + iy, mm)) {
+        kind = geom_kind(I, xx, mm);
+        if (kind == 0) {
+          float gg[5];
+          load_g(mm * nx + xx, gg);
+          phi = gg[0] + ((gg[1] + gg[2]) + (gg[3] + gg[4]));
+        }
+      }
+      solid = solid || kind != 0;
+    }
+    sphi[iy][ix] = phi;
+    skind[iy][ix] = (unsigned char)kind;
+  }
+  const bool any_solid = __syncthreads_or(solid);
+  if (flag & kStatusNumeric) return;  // a lattice whose numeric flag is set is frozen
+  if (any_solid) {
+    // wetting ghosts of the solid cells of two rings (they read fluid cells
+    // only, which stay as they are)
+    for (int k = tid; k < (kCellRX - 2) * (kCellRY - 2); k += kCellThreads) {
+      const int ix = 1 + k % (kCellRX - 2), iy = 1 + k / (kCellRX - 2);
+      const int kd = skind[iy][ix];
+      if (kd == 0) continue;
+#define PK(dx, dy) sphi[iy + (dy)][ix + (dx)], skind[iy + (dy)][ix + (dx)]
+      sphi[iy][ix] = ghost_phi(kd, I.hk, PK(1, 0), PK(0, 1), PK(-1, 0), PK(0, -1), PK(1, 1),
+                               PK(-1, 1), PK(-1, -1), PK(1, -1));
+#undef PK
+    }
+    __syncthreads();
+  }
+  CollK K;
+  K.phis = I.phis;
+  K.inv_phis = I.inv_phis;
+  K.A4 = I.A4;
+  K.kappa = I.kappa;
+  K.omq = I.omq;
+  K.inv_tphi = I.inv_tphi;
+  K.gamma = I.gamma;
+  K.inv2q = I.inv2q;
+  K.qmt = I.q - I.inv_tphi;
+  K.nu_air = I.nu_air;
+  K.dnu = I.dnu;
+  K.n0 = I.n0;
+  K.Fd = drive_at(I, t);
+  float fs[9], gP[4], g0n = 0.0f, n = 0.0f, uy = 0.0f, u2 = 0.0f;
+  const int px = min(cx, nw + 1) + 2, py = min(cy, nh + 1) + 2;  // in the phi region
+  const bool fluid = skind[py][px] == 0;
+  const float phi = fluid ? sphi[py][px] : 0.0f;
+  if (coll) {
+    const bool driven =
+        I.geom != GEOM_NOZZLE || (mapped && m < I.L && x >= I.cx0 && x < I.cx1);
+    collide_cell<false>(fr, g, phi, sphi[py][px], sphi[py][px + 1], sphi[py + 1][px], sphi[py][px - 1],
+                 sphi[py - 1][px], sphi[py + 1][px + 1], sphi[py + 1][px - 1],
+                 sphi[py - 1][px - 1], sphi[py - 1][px + 1], driven, K, fs, gP, g0n, n, uy, u2);
+    if (fluid && !(u2 < 0.09f)) atomicOr(I.status, kStatusNumeric);
+    const int c = cy * kCellCX + cx;
+#pragma unroll
+    for (int i = 1; i < 9; i++) mv[i - 1][c] = fs[i];
+#pragma unroll
+    for (int i = 0; i < 4; i++) mv[8 + i][c] = gP[i];
+  }
+  const bool out = coll && cx >= 1 && cx <= nw && cy >= 1 && cy <= nh;
+  __syncthreads();
+  if (out) {
+    // pull: from the source cell, or, where it is solid, this cell's own
+    // population of the opposite direction (halfway bounce-back)
+    const int c = cy * kCellCX + cx;
+    float f[9], go[5];
+    f[0] = fs[0];
+#pragma unroll
+    for (int i = 1; i < 9; i++) {
+      const int ib = i < 5 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5;  // opposite direction
+      const bool s = skind[py - cEY(i)][px - cEX(i)] != 0;
+      const int from = c - cEY(i) * kCellCX - cEX(i);
+      f[i] = s ? fs[ib] : mv[i - 1][from];
+      if (i < 5) {
+        const float p = s ? gP[ib - 1] : mv[7 + i][from];
+        go[i] = i < 4 ? stay_and_move(K.omq, g[i], p) : stay4(K.omq, g[i]) + p;
+      }
+    }
+    go[0] = g0n;
+    float* __restrict__ fout = I.f[(t + 1) & 1];
+    float* __restrict__ gout = I.g[(t + 1) & 1];
+    __half* __restrict__ fhout = reinterpret_cast<__half*>(fout);
+    __half* __restrict__ ghout = reinterpret_cast<__half*>(gout + N);
+    const int o = (y0 + cy - 1) * nx + x0 + cx - 1;
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+      const float v = fluid ? f[i] : 0.0f;
+      if (H)
+        fhout[(size_t)i * N + o] = __float2half_rn(v);
+      else
+        fout[(size_t)i * N + o] = v;
+    }
+#pragma unroll
+    for (int i = 0; i < 5; i++) {
+      const float v = fluid ? go[i] : 0.0f;
+      if (H && i > 0)
+        ghout[(size_t)(i - 1) * N + o] = __float2half_rn(v);
+      else
+        gout[(size_t)i * N + o] = v;
     }
   }
 }
@@ -1299,6 +1503,39 @@ cudaError_t launch_step(const Inst* d_inst, const Item* d_items, int n_items, in
   if (odd) return diag ? LAUNCH_STEP(true, false, true) : LAUNCH_STEP(false, false, true);
   return diag ? LAUNCH_STEP(true, false, false) : LAUNCH_STEP(false, false, false);
 #undef LAUNCH_STEP
+}
+
+cudaError_t launch_cells(const Inst* d_inst, const Inst* h_inst, int n_inst, const Item* d_items,
+                         int n_items, const long long* d_t, int t_off, bool h16, cudaStream_t s) {
+  if (n_items <= 0) return cudaSuccess;
+#define LAUNCH_CELLS(HH, ON) \
+  cell_kernel<HH, ON><<<n_items, kCellThreads, 0, s>>>(h_inst[0], d_inst, d_items, d_t, t_off)
+  if (h16) {
+    if (n_inst == 1)
+      LAUNCH_CELLS(true, true);
+    else
+      LAUNCH_CELLS(true, false);
+  } else {
+    if (n_inst == 1)
+      LAUNCH_CELLS(false, true);
+    else
+      LAUNCH_CELLS(false, false);
+  }
+#undef LAUNCH_CELLS
+  return cudaGetLastError();
+}
+
+int make_cells(const Inst& I, int k, Item* out, int cap) {
+  int n = 0;
+  for (int y0 = 0; y0 < I.ny; y0 += kCellY)
+    for (int x0 = 0; x0 < I.nx; x0 += kCellX) {
+      if (out) {
+        if (n >= cap) return -1;
+        out[n] = Item{k, x0, std::min(kCellX, I.nx - x0), 0, y0, std::min(kCellY, I.ny - y0), 0, -1};
+      }
+      n++;
+    }
+  return n;
 }
 
 int step_prefetch_for(int) { return 1; }

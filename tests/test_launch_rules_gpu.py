@@ -89,3 +89,35 @@ def test_noalloc_list(ij, nx, ny):
     f1, g1 = ij.ij_get_state(h, 0)
     got = (fo.cpu().numpy().astype(np.float64) + rest).astype(np.float32)
     assert np.array_equal(got, f1) and np.array_equal(go.cpu().numpy(), g1)
+
+
+@pytest.mark.parametrize("ps", [
+    [dict(nx=64, ny=256)], [dict(nx=33, ny=41)], [dict(nx=17, ny=9, axial_bc=1)],
+    [dict(nx=48, ny=96, axial_bc=2)], [dict(nx=50, ny=70, precision=1)],
+    [dict(nx=30, ny=31), dict(nx=64, ny=20, theta_deg=140.0), dict(nx=18, ny=50)],
+    [dict(nx=40, ny=40, plate=1)], [dict(nx=5, ny=7, free=1)], [dict(nx=1, ny=1, free=1)],
+    [dict(nx=400, ny=600)]], ids=str)
+def test_small_lattice_kernel(ij, ps):
+    """The kernel of small lattices against the strip list: the same state bit
+    for bit, through diagnostics steps (every third) and a moving front."""
+    def params(p):
+        q = dict(p)
+        plate, free = q.pop("plate", 0), q.pop("free", 0)
+        nx, ny = q.pop("nx"), q.pop("ny")
+        if plate:
+            return dict(q, nx=nx, ny=ny, geometry=2, wall_thickness=3, axial_bc=2, init_kind=1,
+                        init_x=20.0, init_y=10.0, init_r=9.0, theta_deg=60.0, diag_every=3)
+        if free:
+            return dict(q, nx=nx, ny=ny, init_kind=2, init_y=ny / 2.0, F0=1e-4, T1=100, diag_every=3)
+        w = max(4, nx // 4)
+        return dict(_lat2(nx, ny, **q), nozzle_width=w, wall_thickness=max(1, min(3, (nx - w) // 2)),
+                    diag_every=3)
+    full = [params(p) for p in ps]
+    a, b = ij.ij_create(full), ij.ij_create(full)
+    ij.ij_tune(b, 0, 11, 1)
+    for n in (1, 1, 4, 24):
+        ij.ij_step(a, n)
+        ij.ij_step(b, n)
+    for k in range(len(full)):
+        for u, v in zip(ij.ij_get_state(a, k), ij.ij_get_state(b, k)):
+            assert np.array_equal(u, v), k
