@@ -561,7 +561,6 @@ int default_chunk(ij_handle h, Bucket b) {
 // Measured us a step, in brackets in strips: 64 x 256 4.2 (10.0), 4 x 100 x 400
 // 12.0 (13.7), 400 x 400 10.5 (13.5), 16 x 64 x 256 15.5 (20.7), but 2 x 301 x
 // 501 19.1 (18.0) and 200 x 1600 18.3 (16.8).
-constexpr long long kCellsMost = 240000;
 bool default_cells(ij_handle h) {
   long long cells = 0;
   for (const Inst& I : h->inst) cells += (long long)I.nx * I.ny;

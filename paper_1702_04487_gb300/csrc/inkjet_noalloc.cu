@@ -117,10 +117,6 @@ extern "C" ij_status ij_step_noalloc(const ij_params* params, long long t, const
   int n_items = items_per_lattice(I, kChunk);
   if (n_items > kMaxItems)
     return report(IJ_ERR_PARAM, "ij_step_noalloc: lattice needs more than the fixed 16384 work items");
-  const int strips = (p.nx + kStripCols - 1) / kStripCols;
-  const int rows = (int)std::min<long long>(kChunk, ((long long)strips * p.ny + kSlots - 1) / kSlots);
-  n_items = make_items(I, 0, std::max(2, rows), g_items, kMaxItems);
-  if (n_items < 0) n_items = make_items(I, 0, kChunk, g_items, kMaxItems);
   unsigned char* base = nullptr;
   st = scratch_base(s, &base);
   if (st != IJ_OK) return st;
@@ -134,6 +130,21 @@ extern "C" ij_status ij_step_noalloc(const ij_params* params, long long t, const
   I.hist = reinterpret_cast<double*>(base + kOffHist);
   I.dstate = reinterpret_cast<double*>(base + kOffDstate);
   I.status = reinterpret_cast<unsigned*>(base + kOffStatus);
+  if (!record_out && (long long)p.nx * p.ny <= kCellsMost) {
+    // small lattices, no record: the descriptor and the time come with the
+    // launch, tiles need no list, and the flag is the caller's word if given,
+    // so that nothing is staged on the device (64 x 256: 16 us a call against
+    // 23 with the three copies and strips)
+    if (status_out) I.status = status_out;
+    cudaError_t e = cudaMemsetAsync(I.status, 0, sizeof(unsigned), s);
+    if (e == cudaSuccess)
+      e = launch_cells(nullptr, &I, 1, nullptr, make_cells(I, 0, nullptr, 0), nullptr, t, false, s);
+    return e == cudaSuccess ? IJ_OK : report(IJ_ERR_CUDA, cudaGetErrorString(e));
+  }
+  const int strips = (p.nx + kStripCols - 1) / kStripCols;
+  const int rows = (int)std::min<long long>(kChunk, ((long long)strips * p.ny + kSlots - 1) / kSlots);
+  n_items = make_items(I, 0, std::max(2, rows), g_items, kMaxItems);
+  if (n_items < 0) n_items = make_items(I, 0, kChunk, g_items, kMaxItems);
   const Inst* d_inst = reinterpret_cast<const Inst*>(base + kOffInst);
   const Item* d_items = reinterpret_cast<const Item*>(base + kOffItems);
   long long* d_t = reinterpret_cast<long long*>(base + kOffT);

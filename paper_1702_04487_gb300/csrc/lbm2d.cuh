@@ -57,6 +57,7 @@ struct Item {
 };
 
 constexpr int kStripCols = 60;     // written columns of one work item
+constexpr long long kCellsMost = 240000;  // cells of a handle or call that take launch_cells
 constexpr int kStepThreads = 32;  // one warp per block, one work item each
 constexpr int kStepBlocksPerSM = 10;  // resident blocks per SM the registers are sized for
 constexpr int kMaxPrefetch = 4;    // rows staged ahead of use: 1 .. 4
@@ -90,9 +91,11 @@ cudaError_t launch_step(const Inst* d_inst, const Item* d_items, int n_items, in
                         bool h16, bool odd, cudaStream_t s);
 // The same step, without diagnostics, by the kernel of small lattices: a block per 16 x 8 tile of
 // cells (make_cells: xs, nout, y0, ch of an item are the tile); any nx.
-// h_inst: the descriptors on the host (device pointers inside).
+// h_inst: the descriptors on the host (device pointers inside); of one lattice
+// d_inst and d_items are not read.  d_t null: the time is t_off.
 cudaError_t launch_cells(const Inst* d_inst, const Inst* h_inst, int n_inst, const Item* d_items,
-                         int n_items, const long long* d_t, int t_off, bool h16, cudaStream_t s);
+                         int n_items, const long long* d_t, long long t_off, bool h16,
+                         cudaStream_t s);
 // Tiles of one lattice into out (null: count only); -1 when cap is too small.
 int make_cells(const Inst& I, int k, Item* out, int cap);
 // default number of rows staged ahead of use

@@ -918,7 +918,8 @@ static_assert(kCellCX * kCellCY <= kCellThreads, "a thread per colliding cell");
 template <bool H, bool ONE>
 __global__ void __launch_bounds__(kCellThreads)
     cell_kernel(const __grid_constant__ Inst one, const Inst* __restrict__ insts,
-                const Item* __restrict__ items, const long long* __restrict__ d_t, int t_off) {
+                const Item* __restrict__ items, const long long* __restrict__ d_t,
+                long long t_off) {
   __shared__ float sphi[kCellRY][kCellRX];
   __shared__ unsigned char skind[kCellRY][kCellRX];
   __shared__ float mv[12][kCellCY * kCellCX];  // f*_1..8, moving g_1..4
@@ -936,7 +937,7 @@ __global__ void __launch_bounds__(kCellThreads)
   const Inst& I = ONE ? one : insts[it.inst];
   const int tid = threadIdx.x;
   if (tid == 0) flag = *(volatile const unsigned*)I.status;
-  const long long t = *d_t + t_off;
+  const long long t = (d_t ? *d_t : 0) + t_off;
   const int nx = I.nx, N = nx * I.ny, x0 = it.xs, y0 = it.y0, nw = it.nout, nh = it.ch;
   const float* __restrict__ fin = I.f[t & 1];
   const float* __restrict__ gin = I.g[t & 1];
@@ -1506,7 +1507,8 @@ cudaError_t launch_step(const Inst* d_inst, const Item* d_items, int n_items, in
 }
 
 cudaError_t launch_cells(const Inst* d_inst, const Inst* h_inst, int n_inst, const Item* d_items,
-                         int n_items, const long long* d_t, int t_off, bool h16, cudaStream_t s) {
+                         int n_items, const long long* d_t, long long t_off, bool h16,
+                         cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
 #define LAUNCH_CELLS(HH, ON) \
   cell_kernel<HH, ON><<<n_items, kCellThreads, 0, s>>>(h_inst[0], d_inst, d_items, d_t, t_off)
