@@ -630,8 +630,8 @@ ij_status check_handle(ij_handle h) {
 }
 
 // One 3-D time step on stream s (time d_t[0] + t_off): the fused step of
-// every lattice (with plane sums when diag), the wetting ghosts of the new
-// phi, the flip of the current buffers.  The diagnostics record is the
+// every lattice (with plane sums when diag), then the derived entries of the
+// new phi and the flip of the current buffers.  The diagnostics record is the
 // caller's.
 cudaError_t enqueue_step3(ij_handle h, cudaStream_t s, int t_off, bool diag, long long* n) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -650,9 +650,6 @@ cudaError_t enqueue_step3(ij_handle h, cudaStream_t s, int t_off, bool diag, lon
   }
   if (e != cudaSuccess) return e;
   e = launch_ghost3(h->d_inst3, h->inst3.data(), h->n_inst, true, s);
-  (*n)++;
-  if (e != cudaSuccess) return e;
-  e = launch_flip3(h->d_inst3, h->n_inst, s);
   (*n)++;
   return e;
 }
@@ -830,7 +827,7 @@ ij_status create3(ij_handle h) {
   if (e3 != cudaSuccess) return fail(IJ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e3));
   h->inst3.resize(count);
   h->inst.resize(count);
-  std::vector<int> ghosts;
+  std::vector<int2> ghosts;
   for (int k = 0; k < count; k++) {
     const ij_params& p = h->params[k];
     Inst3 I = derive3(p);
@@ -845,12 +842,12 @@ ij_status create3(ij_handle h) {
       if (!I.f[b] || !I.g[b] || !I.g0[b] || !I.phi[b])
         return fail(IJ_ERR_OOM, "device allocation of 3-D lattice %d failed", k);
     }
-    I.n_ghost = ghost_cells3(I, nullptr);
+    I.n_ghost = derived_phi3(I, nullptr);
     ghosts.resize(std::max(1, I.n_ghost));
-    ghost_cells3(I, ghosts.data());
-    I.ghost = (int*)h->dalloc(ghosts.size() * sizeof(int));
+    derived_phi3(I, ghosts.data());
+    I.ghost = (int2*)h->dalloc(ghosts.size() * sizeof(int2));
     if (!I.ghost) return fail(IJ_ERR_OOM, "device allocation of 3-D lattice %d failed", k);
-    CUDA_TRY(cudaMemcpyAsync(I.ghost, ghosts.data(), ghosts.size() * sizeof(int),
+    CUDA_TRY(cudaMemcpyAsync(I.ghost, ghosts.data(), ghosts.size() * sizeof(int2),
                              cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));  // ghosts is reused
     // the step never stores solid cells: they hold 0 in both buffers
@@ -884,12 +881,13 @@ ij_status create3(ij_handle h) {
   h->d_inst = (Inst*)h->dalloc(count * sizeof(Inst));
   h->d_t = (long long*)h->dalloc(sizeof(long long));
   h->d_status = (unsigned*)h->dalloc(count * sizeof(unsigned));
-  int* d_cur = (int*)h->dalloc(count * sizeof(int));
+  int* d_cur = (int*)h->dalloc(2 * (size_t)count * sizeof(int));
   if (!h->d_inst3 || !h->d_inst || !h->d_t || !h->d_status || !d_cur)
     return fail(IJ_ERR_OOM, "device allocation of descriptors failed");
   for (int k = 0; k < count; k++) {
     h->inst3[k].status = h->inst[k].status = h->d_status + k;
     h->inst3[k].cur = d_cur + k;
+    h->inst3[k].done = d_cur + count + k;
   }
   if (cudaMallocHost((void**)&h->h_status, count * sizeof(unsigned)) != cudaSuccess)
     return fail(IJ_ERR_OOM, "pinned allocation failed");
@@ -905,7 +903,7 @@ ij_status create3(ij_handle h) {
   CUDA_TRY(cudaMemcpyAsync(h->d_inst, h->inst.data(), count * sizeof(Inst), cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemsetAsync(h->d_t, 0, sizeof(long long), s));
   CUDA_TRY(cudaMemsetAsync(h->d_status, 0, count * sizeof(unsigned), s));
-  CUDA_TRY(cudaMemsetAsync(d_cur, 0, count * sizeof(int), s));
+  CUDA_TRY(cudaMemsetAsync(d_cur, 0, 2 * (size_t)count * sizeof(int), s));
   const double dinit[8] = {0, 0, 0, -1, 0, 0, 0, 0};
   for (int k = 0; k < count; k++) {
     const Inst& D = h->inst[k];

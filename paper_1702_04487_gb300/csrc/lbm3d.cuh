@@ -34,8 +34,12 @@ struct Inst3 {
   void* g[2];
   float* g0[2];
   float* phi[2];
-  int* ghost;    // [n_ghost]: in-domain solid cells within reach of a fluid stencil
+  // [n_ghost] {index in phi, fluid neighbours}: the entries of phi derived
+  // after each step (in-domain solid cells within reach of a fluid stencil,
+  // the four extended planes)
+  int2* ghost;
   int* cur;      // index of the buffer holding the current state
+  int* done;     // blocks that have finished (ghost3_kernel), zero between launches
   double* rows;  // [3][nz]
   double* sums;  // [4]
   unsigned* status;
@@ -51,10 +55,9 @@ struct Item3 {
 constexpr int kTile3X = 28, kTile3Y = 12;  // written columns of a 3-D work item
 constexpr int kStep3Threads = 512;          // threads of a step3 CTA (32 x 16 columns)
 
-// Solid cells of lattice h within reach of a fluid D3Q19 stencil (cell
-// indices z * ny * nx + y * nx + x), written to out when not null; returns
-// their number.  Host code.
-int ghost_cells3(const Inst3& h, int* out);
+// The derived entries of phi (Inst3::ghost), written to out when not null;
+// returns their number.  Host code.
+int derived_phi3(const Inst3& h, int2* out);
 // Work items of every lattice into out (null: count only); returns the count.
 int make_items3(const Inst3* h, int n_inst, int chunk, Item3* out);
 
@@ -63,11 +66,10 @@ cudaError_t launch_init3(const Inst3* d_inst, const Inst3& h, int index, cudaStr
 // t_off, from buffer *cur into the other one
 cudaError_t launch_step3(const Inst3* d_inst, const Item3* d_items, int n_items, int n_inst,
                          const long long* d_t, int t_off, bool diag, bool h16, cudaStream_t s);
-// wetting ghosts and extended planes of phi in buffer *cur (next: the other
-// buffer, which the step just wrote)
+// derived entries of phi in buffer *cur (next: in the other buffer, which the
+// step just wrote and which then becomes current, for every lattice that is
+// not frozen)
 cudaError_t launch_ghost3(const Inst3* d_inst, const Inst3* h, int n_inst, bool next, cudaStream_t s);
-// *cur ^= 1 for every lattice that is not frozen
-cudaError_t launch_flip3(const Inst3* d_inst, int n_inst, cudaStream_t s);
 // state (current buffer) <-> absolute FP32 populations f[19][N], g[7][N]
 // (solid cells 0); import also refreshes phi with its ghosts
 cudaError_t launch_export3(const Inst3* d_inst, const Inst3& h, int index, float* f, float* g,
