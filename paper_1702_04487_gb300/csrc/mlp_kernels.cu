@@ -127,6 +127,26 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int j = 0; j < 16; j++) v[j] = __uint_as_float(r[j]);
 }
 
+// The two halves of it: start the load, and wait for every load started (the
+// values pass through the wait, so nothing reads them before it).
+__device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+      "%14,%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld16_wait(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                 "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+
 // The same for 8 columns.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
   uint32_t r[8];
@@ -479,15 +499,9 @@ __global__ void cast_params_kernel(const float* __restrict__ p, const Layout L, 
 // tensor-memory lanes 32 (w mod 4) .. + 31 and every (warps / 4)-th group of
 // 16 units.
 //
-// Bound by the GELUs (an erff each: 4 H per query and member) at instruction
-// issue; two CTAs of 256 threads share an SM, so one's tensor-core pass and
-// weight loads run beside the other's GELUs.  While the grid has at most one
-// tile per SM, one CTA of 512 threads and a ring of nine chunks per SM halve
-// the serial chain of a layer instead.  Measured, five members of H = 256:
-// 65536 queries 500 us, against 2190 us for a GEMM launch per layer with the
-// activations through HBM (the same results, bit for bit).
+// Bound by latency here (up to a tile per SM); many tiles take pair_kernel.
 constexpr int kFwdChunk = 128 * BK * 2;  // bytes of a weight chunk, and of 64 activation columns
-constexpr int kFwdRingMax = 9;
+constexpr int kFwdRing = 9;
 
 struct FwdMaps {
   CUtensorMap w[kHidden + 1];  // boxes of 64 (K) x 128 (units) x 1 (member)
@@ -503,10 +517,7 @@ struct FwdArgs {
   unsigned* status;
 };
 
-template <int NT>
-__host__ __device__ constexpr int fwd_ring() {
-  return NT == 256 ? 3 : kFwdRingMax;
-}
+constexpr int kFwdThreads = 512;
 // activations, ring, then the barriers and the tensor-memory address (no
 // static shared memory: the dynamic part then starts on a 1024-byte boundary
 // and two CTAs of H = 256 fit an SM)
@@ -515,11 +526,10 @@ size_t fwd_smem_bytes(int H, int ring) {
   return (size_t)((H + BK - 1) / BK + ring) * kFwdChunk + kFwdTail;
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
+__global__ void __launch_bounds__(kFwdThreads, 1)
     forward_kernel(const __grid_constant__ FwdMaps maps, const FwdArgs a) {
   extern __shared__ __align__(1024) uint8_t fwd_smem[];
-  constexpr int R = fwd_ring<NT>();
+  constexpr int R = kFwdRing, NT = kFwdThreads;
   const int H = a.H, slices = (H + BK - 1) / BK;
   uint8_t* const smem = fwd_smem;
   uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + (size_t)(slices + R) * kFwdChunk);
@@ -682,6 +692,230 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(cols)
+                 : "memory");
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Inference of many queries: the same on two 128-row tiles per CTA, one CTA
+// per SM.  16 warps do nothing but output passes, alternating between the
+// tiles; a warp each issues the products and loads the weights (streamed from
+// L2 once per tile and layer through a ring of 16 KB chunks).  While the
+// output pass of one tile runs, the tensor cores work on the other, so that
+// the instruction issue, which bounds this kernel, never waits for them.
+//  ready[t]: the 16 warps have written tile t's next operand and are done with
+//  its accumulator; done[t]: its products are complete.
+//
+// Bound by the GELUs (an erff each: 4 H per query and member, 32 instructions
+// a GELU) at instruction issue.  Measured, five members of H = 256: a call of
+// 65536 queries takes 534 us, 619 with a tile per CTA and two CTAs per SM (56 %
+// issue: both wait for their products together), 568 without the accumulator
+// loads one step ahead, and 2190 us more for a GEMM launch per layer with the
+// activations through HBM.
+constexpr int kPairRing = 6;
+constexpr int kPairWarps = 16;
+constexpr int kPairThreads = (kPairWarps + 2) * 32;
+size_t pair_smem_bytes(int H) {
+  return (size_t)(2 * ((H + BK - 1) / BK) + kPairRing) * kFwdChunk + kFwdTail;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+
+__global__ void __launch_bounds__(kPairThreads, 1)
+    pair_kernel(const __grid_constant__ FwdMaps maps, const FwdArgs a) {
+  extern __shared__ __align__(1024) uint8_t fwd_smem[];
+  constexpr int R = kPairRing;
+  const int H = a.H, slices = (H + BK - 1) / BK;
+  const uint32_t base = smem_u32(fwd_smem), blk = (uint32_t)slices * kFwdChunk;
+  const uint32_t ring = base + 2 * blk, tail = ring + R * kFwdChunk;
+  const uint32_t b_full = tail, b_empty = tail + 8 * R, b_ready = tail + 16 * R,
+                 b_done = b_ready + 16;
+  uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(fwd_smem + (tail - base) + 16 * R + 32);
+  static_assert(16 * R + 36 <= kFwdTail, "barriers outgrew their slot");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.x * 2 * BM, z = blockIdx.y;
+  const uint32_t cols = H <= 32 ? 32 : H <= 64 ? 64 : H <= 128 ? 128 : 256;  // of one tile
+  const int tiles = m0 + BM < a.n ? 2 : 1;
+  if (tid == 0) {
+#pragma unroll
+    for (int i = 0; i < 2 * R; i++) mbar_init(b_full + 8 * i, 1);
+#pragma unroll
+    for (int t = 0; t < 2; t++) {
+      mbar_init(b_ready + 8 * t, kPairWarps);
+      mbar_init(b_done + 8 * t, 1);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(2 * cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *(volatile uint32_t*)tmem_slot;
+  auto units_of = [&](int l) { return l < kHidden ? H : kOutPad; };
+  auto depth_of = [&](int l) { return l == 0 ? kInPad : H; };
+  bool ok = true;
+  if (warp == kPairWarps + 1) {
+    // the weights: every layer's chunks, K slice by K slice, 128 output units
+    // at a time, once per tile
+    if (lane == 0) {
+      int c = 0;
+      for (int l = 0; l <= kHidden && ok; l++)
+        for (int t = 0; t < tiles && ok; t++)
+          for (int s = 0; s * BK < depth_of(l) && ok; s++)
+            for (int h = 0; h * 128 < units_of(l); h++) {
+              const int b = c % R;
+              if (c >= R && !mbar_wait(b_empty + 8 * b, (uint32_t)((c / R - 1) & 1))) {
+                ok = false;
+                break;
+              }
+              mbar_expect_tx(b_full + 8 * b, (uint32_t)kFwdChunk);
+              tma_load3(ring + (uint32_t)b * kFwdChunk, &maps.w[l], s * BK, h * 128, z, b_full + 8 * b);
+              c++;
+            }
+      // no copy may land after the CTA ends (bounded)
+      if (!ok)
+        for (int k = c > R ? c - R : 0; k < c; k++)
+          mbar_wait(b_full + 8 * (k % R), (uint32_t)((k / R) & 1));
+    }
+    __syncwarp();
+  } else if (warp == kPairWarps) {
+    if (lane == 0) {
+      int c = 0;
+      for (int l = 0; l <= kHidden && ok; l++)
+        for (int t = 0; t < tiles && ok; t++) {
+          if (!mbar_wait(b_ready + 8 * t, (uint32_t)(l & 1))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const int K = depth_of(l), N = units_of(l);
+          for (int s = 0; s * BK < K && ok; s++)
+            for (int h = 0; h * 128 < N; h++) {
+              const int b = c % R;
+              if (!mbar_wait(b_full + 8 * b, (uint32_t)((c / R) & 1))) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const int nn = N - h * 128 < 128 ? N - h * 128 : 128;
+              const int steps = K - s * BK < BK ? (K - s * BK) / 16 : BK / 16;
+              const uint64_t da = sw128_desc(base + t * blk + (uint32_t)s * kFwdChunk);
+              const uint64_t db = sw128_desc(ring + (uint32_t)b * kFwdChunk);
+              const uint32_t id = idesc_bf16(BM, nn);
+              for (int k = 0; k < steps; k++)
+                mma_bf16(tmem + t * cols + h * 128, da + 2u * k, db + 2u * k, id,
+                         (s > 0 || k > 0) ? 1u : 0u);
+              mma_commit(b_empty + 8 * b);
+              c++;
+            }
+          mma_commit(b_done + 8 * t);
+        }
+      // no MMA may run after the CTA ends (bounded)
+      if (!ok)
+        for (int k = c > R ? c - R : 0; k < c; k++)
+          mbar_wait(b_empty + 8 * (k % R), (uint32_t)((k / R) & 1));
+    }
+    __syncwarp();
+  } else {
+    // layer 0's operands: transformed queries, BF16, columns 7..15 zero
+    if (tid < 2 * BM) {
+      const int row = m0 + tid, r = tid & (BM - 1);
+      __align__(16) bf16 v[kInPad];
+#pragma unroll
+      for (int d = 0; d < kInPad; d++)
+        v[d] = __float2bfloat16_rn(
+            d < kIn && row < a.n ? xform(a.x[(size_t)row * kIn + d], d, a.xf) : 0.0f);
+#pragma unroll
+      for (int c = 0; c < 2; c++)
+        *reinterpret_cast<uint4*>(fwd_smem + (tid >> 7) * blk + r * 128 + ((c ^ (r & 7)) << 4)) =
+            reinterpret_cast<const uint4*>(v)[c];
+    }
+    // this warp is done with tile t: its stores are visible to the tensor
+    // cores, its reads of the accumulator complete
+    auto hand_over = [&](int t) {
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_ready + 8 * t);
+    };
+    for (int t = 0; t < tiles; t++) hand_over(t);
+    for (int l = 0; l <= kHidden && ok; l++)
+      for (int t = 0; t < tiles; t++) {
+        if (!mbar_wait(b_done + 8 * t, (uint32_t)(l & 1))) {
+          ok = false;
+          break;
+        }
+        __syncwarp();
+        tc_fence_after();
+        const int mt = m0 + t * BM, r = (warp & 3) * 32 + lane;
+        const uint32_t acc = tmem + t * cols + ((uint32_t)((warp & 3) * 32) << 16);
+        const bool rows_in = mt + (warp & 3) * 32 < a.n;  // any valid row of this warp's 32
+        const float* bias = a.p + z * a.P + a.b_off[l];
+        if (l < kHidden) {
+          if (rows_in) {
+            // the accumulator's next 16 columns are on their way while these
+            // are worked on
+            constexpr int kStep = kPairWarps / 4 * 16;
+            auto work = [&](int c0, const uint32_t (&v)[16]) {
+              __align__(16) bf16 o[16];
+#pragma unroll
+              for (int j = 0; j < 16; j += 4) {
+                const float4 b4 = __ldg(reinterpret_cast<const float4*>(bias + c0 + j));
+                o[j] = __float2bfloat16_rn(gelu_f(__uint_as_float(v[j]) + b4.x));
+                o[j + 1] = __float2bfloat16_rn(gelu_f(__uint_as_float(v[j + 1]) + b4.y));
+                o[j + 2] = __float2bfloat16_rn(gelu_f(__uint_as_float(v[j + 2]) + b4.z));
+                o[j + 3] = __float2bfloat16_rn(gelu_f(__uint_as_float(v[j + 3]) + b4.w));
+              }
+              const int ch = (c0 % BK) / 8;
+              uint8_t* row = fwd_smem + t * blk + (size_t)(c0 / BK) * kFwdChunk + r * 128;
+#pragma unroll
+              for (int c = 0; c < 2; c++)
+                *reinterpret_cast<uint4*>(row + (((ch + c) ^ (r & 7)) << 4)) =
+                    reinterpret_cast<const uint4*>(o)[c];
+            };
+            uint32_t va[16], vb[16];
+            int c0 = (warp >> 2) * 16;
+            if (c0 < H) tmem_ld16_start(acc + (uint32_t)c0, va);
+#pragma unroll 1
+            for (; c0 < H; c0 += 2 * kStep) {
+              tmem_ld16_wait(va);
+              if (c0 + kStep < H) tmem_ld16_start(acc + (uint32_t)(c0 + kStep), vb);
+              work(c0, va);
+              if (c0 + kStep >= H) break;
+              tmem_ld16_wait(vb);
+              if (c0 + 2 * kStep < H) tmem_ld16_start(acc + (uint32_t)(c0 + 2 * kStep), va);
+              work(c0 + kStep, vb);
+            }
+          }
+          hand_over(t);
+        } else if (warp < 4 && rows_in) {
+          float v[16];
+          tmem_ld16(acc, v);
+          const int row = mt + r;
+          if (row < a.n)
+            *reinterpret_cast<float4*>(a.Y + ((size_t)z * a.n + row) * kOut) =
+                make_float4(v[0] + __ldg(bias), v[1] + __ldg(bias + 1), v[2] + __ldg(bias + 2),
+                            v[3] + __ldg(bias + 3));
+        }
+      }
+  }
+  if (!ok && lane == 0) atomicOr(a.status, kStatusTimeout);
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
+                 "r"(2 * cols)
                  : "memory");
   }
 }
@@ -1542,18 +1776,18 @@ cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* 
   }
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(forward_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fwd_smem_bytes(256, fwd_ring<256>()));
+    cudaError_t e = cudaFuncSetAttribute(forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)fwd_smem_bytes(256, kFwdRing));
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(forward_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)fwd_smem_bytes(256, fwd_ring<512>()));
+      e = cudaFuncSetAttribute(pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)pair_smem_bytes(256));
     if (e != cudaSuccess) return e;
     attr = true;
   }
   if ((long long)grid.x * grid.y <= 152)  // at most one tile per SM
-    forward_kernel<512><<<grid, 512, fwd_smem_bytes(a.H, fwd_ring<512>()), s>>>(maps, a);
+    forward_kernel<<<grid, kFwdThreads, fwd_smem_bytes(a.H, kFwdRing), s>>>(maps, a);
   else
-    forward_kernel<256><<<grid, 256, fwd_smem_bytes(a.H, fwd_ring<256>()), s>>>(maps, a);
+    pair_kernel<<<dim3(blocks(n, 2 * BM), members), kPairThreads, pair_smem_bytes(a.H), s>>>(maps, a);
   return cudaGetLastError();
 }
 
