@@ -73,16 +73,22 @@ __device__ __forceinline__ void stS(void* p, unsigned i, float v) {
 // read again only in the next step, so its lines should not push the current
 // state's planes, which neighbouring tiles still read, out of L2.
 template <bool H>
-__device__ __forceinline__ void stCS(void* p, unsigned i, float v) {
+__device__ __forceinline__ void stCS(void* p, float v) {
   if (H) {
     const __half h = __float2half_rn(v);
-    asm volatile("st.global.cs.b16 [%0], %1;\n" ::"l"(reinterpret_cast<__half*>(p) + i),
-                 "h"(__half_as_ushort(h))
-                 : "memory");
+    asm volatile("st.global.cs.b16 [%0], %1;\n" ::"l"(p), "h"(__half_as_ushort(h)) : "memory");
   } else {
-    asm volatile("st.global.cs.f32 [%0], %1;\n" ::"l"(reinterpret_cast<float*>(p) + i), "f"(v)
-                 : "memory");
+    asm volatile("st.global.cs.f32 [%0], %1;\n" ::"l"(p), "f"(v) : "memory");
   }
+}
+// p + i * stride bytes, one wide multiply-add (a 32-bit index i * N + c per
+// access took a second instruction: 52 of the 780 of a cell and plane; 2 x 128 x
+// 128 x 640, a step: 1317 -> 1285 us in FP32 storage, 1244 -> 1204 in FP16).
+__device__ __forceinline__ char* at(void* p, unsigned stride, int i) {
+  return static_cast<char*>(p) + (unsigned long long)stride * (unsigned)i;
+}
+__device__ __forceinline__ const char* at(const void* p, unsigned stride, int i) {
+  return static_cast<const char*>(p) + (unsigned long long)stride * (unsigned)i;
 }
 // The value stS stores, as read back later.
 template <bool H>
@@ -470,26 +476,25 @@ __global__ void __launch_bounds__(kThreads3, 1)
     // and the next; nx is even, so pairs never straddle the wrap).
     auto stage = [&](bool in, int zm, int sl, bool need) {
       if (need && in) {
-        const unsigned N = (unsigned)ctx->plane * (unsigned)ctx->nz;
+        constexpr unsigned es = H ? 2 : 4;
+        const unsigned Nb = (unsigned)ctx->plane * (unsigned)ctx->nz * es;
         const unsigned c = cell_of(zm);
         const unsigned d = mypop_a + sl * (S::PW * 4);
+        const char* f = static_cast<const char*>(ctx->fin) + (size_t)c * es;
+        const char* g = static_cast<const char*>(ctx->gin) + (size_t)c * es;
         if (!H) {
-          const float* f = static_cast<const float*>(ctx->fin);
-          const float* g = static_cast<const float*>(ctx->gin);
 #pragma unroll
-          for (int i = 0; i < 19; i++) cp4_async(d + (i * 32 + lane) * 4, f + (c + i * N));
+          for (int i = 0; i < 19; i++) cp4_async(d + (i * 32 + lane) * 4, at(f, Nb, i));
           cp4_async(d + (19 * 32 + lane) * 4, ctx->g0in + c);
 #pragma unroll
-          for (int i = 0; i < 6; i++) cp4_async(d + ((20 + i) * 32 + lane) * 4, g + (c + i * N));
+          for (int i = 0; i < 6; i++) cp4_async(d + ((20 + i) * 32 + lane) * 4, at(g, Nb, i));
         } else {
-          const __half* f = static_cast<const __half*>(ctx->fin);
-          const __half* g = static_cast<const __half*>(ctx->gin);
           cp4_async(d + (304 + lane) * 4, ctx->g0in + c);
           if ((lane & 1) == 0) {
 #pragma unroll
-            for (int i = 0; i < 19; i++) cp4_async(d + (i * 16 + (lane >> 1)) * 4, f + (c + i * N));
+            for (int i = 0; i < 19; i++) cp4_async(d + (i * 16 + (lane >> 1)) * 4, at(f, Nb, i));
 #pragma unroll
-            for (int i = 0; i < 6; i++) cp4_async(d + (336 + i * 16 + (lane >> 1)) * 4, g + (c + i * N));
+            for (int i = 0; i < 6; i++) cp4_async(d + (336 + i * 16 + (lane >> 1)) * 4, at(g, Nb, i));
           }
         }
       }
@@ -704,15 +709,19 @@ __global__ void __launch_bounds__(kThreads3, 1)
           if (written && !sol(smPrev, 0, 0)) {
             const int zo = Zc - 1;
             const float g6 = gs6 + p6;
-            const unsigned N = (unsigned)ctx->plane * (unsigned)ctx->nz, c = cell_of(zo);
-            stCS<H>(ctx->fout, 6 * N + c, f6);
-            stCS<H>(ctx->fout, 13 * N + c, f13);
-            stCS<H>(ctx->fout, 14 * N + c, f14);
-            stCS<H>(ctx->fout, 17 * N + c, f17);
-            stCS<H>(ctx->fout, 18 * N + c, f18);
-            stCS<H>(ctx->gout, 5 * N + c, g6);
+            constexpr unsigned es = H ? 2 : 4;
+            const unsigned Nb = (unsigned)ctx->plane * (unsigned)ctx->nz * es, c = cell_of(zo);
+            char* const f = static_cast<char*>(ctx->fout) + (size_t)c * es;
+            char* const g = static_cast<char*>(ctx->gout) + (size_t)c * es;
+            float* const ph = ctx->phout + (c + 2u * (unsigned)ctx->plane);
+            stCS<H>(at(f, Nb, 6), f6);
+            stCS<H>(at(f, Nb, 13), f13);
+            stCS<H>(at(f, Nb, 14), f14);
+            stCS<H>(at(f, Nb, 17), f17);
+            stCS<H>(at(f, Nb, 18), f18);
+            stCS<H>(at(g, Nb, 5), g6);
             // phi of the new state as the next step sums it (stored values)
-            stCS<false>(ctx->phout, c + 2u * (unsigned)ctx->plane, pg0 + (pg14 + (pg5 + stored<H>(g6))));
+            stCS<false>(ph, pg0 + (pg14 + (pg5 + stored<H>(g6))));
           }
         }
         // ---- gather the pulls of plane Zc (rest, in-plane movers, upward
@@ -746,15 +755,19 @@ __global__ void __launch_bounds__(kThreads3, 1)
           // every pull of plane Zc but f_6, f_13, f_14, f_17, f_18 and the
           // moving part of g_6 is complete: store it now
           if (written && k >= 1 && k <= ch && fluidC) {
-            const unsigned N = (unsigned)ctx->plane * (unsigned)ctx->nz, c = cell_of(Zc);
+            constexpr unsigned es = H ? 2 : 4;
+            const unsigned Nb = (unsigned)ctx->plane * (unsigned)ctx->nz * es, c = cell_of(Zc);
+            char* const f = static_cast<char*>(ctx->fout) + (size_t)c * es;
+            char* const g = static_cast<char*>(ctx->gout) + (size_t)c * es;
+            float* const g0 = ctx->g0out + c;
             const float fo[14] = {fs[0], f1, f2, f3, f4, f5, f7, f8, f9, f10, f11, f12, f15, f16};
             constexpr int fi[14] = {0, 1, 2, 3, 4, 5, 7, 8, 9, 10, 11, 12, 15, 16};
 #pragma unroll
-            for (int j = 0; j < 14; j++) stCS<H>(ctx->fout, fi[j] * N + c, fo[j]);
+            for (int j = 0; j < 14; j++) stCS<H>(at(f, Nb, fi[j]), fo[j]);
             const float go[6] = {g0n, gS[0] + q1, gS[1] + q2, gS[2] + q3, gS[3] + q4, gS[4] + q5};
-            stCS<false>(ctx->g0out, c, go[0]);
+            stCS<false>(g0, go[0]);
 #pragma unroll
-            for (int j = 1; j < 6; j++) stCS<H>(ctx->gout, (j - 1) * N + c, go[j]);
+            for (int j = 1; j < 6; j++) stCS<H>(at(g, Nb, j - 1), go[j]);
             pg0 = go[0];
             pg14 = (stored<H>(go[1]) + stored<H>(go[2])) + (stored<H>(go[3]) + stored<H>(go[4]));
             pg5 = stored<H>(go[5]);
