@@ -1060,6 +1060,9 @@ __global__ void __launch_bounds__(kChainThreads, 1)
       *reinterpret_cast<uint4*>(fwd_smem + (s - base) + tid * 64 + ((c ^ ((tid >> 1) & 3)) << 4)) =
           reinterpret_cast<const uint4*>(v)[c];
   };
+  // rows taken in order were prepared by the kernels just before; the training
+  // rows and the step are constant during a call and need no wait
+  if (TRAIN && a.direct) wait_for_previous();
   // layer 0's operand (every CTA for itself), BF16, columns 7..15 zero
   const int row = m0 + (tid & 127);
   const bool row_in = row < a.rows;
@@ -1071,14 +1074,14 @@ __global__ void __launch_bounds__(kChainThreads, 1)
       if (row_in) {
         int src = row;
         if (!a.direct) {
-          const unsigned long long ctr = ((unsigned long long)z << 56) ^
-                                         ((unsigned long long)(*a.d_step + a.step_off) << 24) ^
-                                         (unsigned)row;
+          const unsigned long long ctr =
+              ((unsigned long long)z << 56) ^
+              ((unsigned long long)(__ldcg(a.d_step) + a.step_off) << 24) ^ (unsigned)row;
           src = (int)(mix64(a.seed ^ mix64(ctr)) % (unsigned long long)a.n);
         }
-        q[0] = reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad)[0];
-        q[1] = reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad)[1];
-        const float4 t4 = reinterpret_cast<const float4*>(a.T)[src];
+        q[0] = __ldcg(reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad));
+        q[1] = __ldcg(reinterpret_cast<const uint4*>(a.X + (size_t)src * kInPad) + 1);
+        const float4 t4 = __ldcg(reinterpret_cast<const float4*>(a.T) + src);
         target[0] = t4.x;
         target[1] = t4.y;
         target[2] = t4.z;
@@ -1093,9 +1096,8 @@ __global__ void __launch_bounds__(kChainThreads, 1)
     }
     put_row(base, v0);
   }
-  // Up to here nothing depends on the kernel before (the training rows and
-  // the step are constant during a call).  From here on: its parameters; and
-  // it has finished reading what this one overwrites.
+  // Up to here nothing depends on the kernel before.  From here on: its
+  // parameters; and it has finished reading what this one overwrites.
   if (TRAIN) {
     wait_for_previous();
     let_next_start();
@@ -1374,11 +1376,12 @@ struct AdamStep {
 // elementary functions on the IBM RISC System/6000", 1990, theorem on
 // quotients from a correctly rounded reciprocal).  The remainder is exact
 // while it does not underflow; moments below 1e-30, where it may, are far
-// below eps in Adam's denominator.  The general division takes a range check
-// and a branch each, a fifth of this kernel's instructions.
+// below eps in Adam's denominator; an infinite quotient stays infinite.  The
+// general division takes a range check and a branch each, a fifth of this
+// kernel's instructions.
 __device__ __forceinline__ float quotient(float a, float b, float y) {
   const float q = __fmul_rn(a, y);
-  return fmaf(fmaf(-q, b, a), y, q);
+  return fabsf(q) < INFINITY ? fmaf(fmaf(-q, b, a), y, q) : q;
 }
 
 // One parameter: moments, update; returns the new value.
@@ -1426,9 +1429,11 @@ __global__ void __launch_bounds__(kUpdateThreads, 1)
   }
   AdamStep s{a.lr, 1.0f, 1.0f, 1.0f, 1.0f};
   if (!a.grads_only) {
-    const long long step = *a.d_step + a.step_off;
-    if (a.d_sched && a.d_sched[1] > 0) {
-      const float frac = (float)(step - a.d_sched[0]) / (float)a.d_sched[1];
+    const long long step = __ldcg(a.d_step) + a.step_off;
+    const long long first = a.d_sched ? __ldcg(a.d_sched) : 0;
+    const long long steps = a.d_sched ? __ldcg(a.d_sched + 1) : 0;
+    if (steps > 0) {
+      const float frac = (float)(step - first) / (float)steps;
       s.lr *= 0.5f * (1.0f + cospif(fminf(fmaxf(frac, 0.0f), 1.0f)));
     }
     const float t = (float)(step + 1);
