@@ -302,7 +302,7 @@ def run_native(args):
         inkjet.ij_tune(h, 0, chunk, pf)
         tuning = inkjet.ij_get_tuning(h)
     else:
-        # 3-D: the default z chunk (80 planes); the tuner's candidates differ
+        # 3-D: the untuned z chunk; the tuner's candidates differ
         # by a few per cent there and its pick varies from run to run
         tune = args.autotune and params[0].get("dim", 2) != 3
         tuning = inkjet.ij_autotune(h, 3) if tune else inkjet.ij_get_tuning(h)

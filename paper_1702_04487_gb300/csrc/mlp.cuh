@@ -1,6 +1,6 @@
 // Internal declarations of the surrogate network's kernels (BF16 tensor-core
-// GEMM with fused epilogues, loss, bias gradients, Adam, input/output
-// transforms, the acceptance gate).  Shared by mlp_kernels.cu and the host
+// GEMM, training step, inference, input transforms, the acceptance gate).
+// Shared by mlp_kernels.cu and the host
 // API in surrogate_api.cu.
 #pragma once
 #include <cuda_bf16.h>

@@ -1,8 +1,8 @@
-// Kernels of the surrogate network: a BF16 tensor-core GEMM on the 5th
-// generation tensor cores (tcgen05.mma, accumulator in tensor memory) with
-// fused epilogues, and the small element-wise kernels around it (input
-// transform and minibatch gather, loss, bias gradients, Adam, output
-// transform, acceptance gate).
+// Kernels of the surrogate network on the 5th generation tensor cores
+// (tcgen05.mma, accumulator in tensor memory): a plain BF16 GEMM and, built
+// from the same pieces, the training step (chain_kernel, update_kernel), the
+// inference kernels (chain_kernel, forward_kernel, pair_kernel) and the answer
+// kernel (decoding, ensemble spread, acceptance gate).
 //
 // GEMM shape: C[M x N] = A[M x K] B[N x K]^T with A and B row-major (K
 // contiguous, "K-major").  A CTA of 128 threads owns a 128 x BN tile of C,
@@ -413,7 +413,7 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t s) {
 }  // namespace sg
 
 // ---------------------------------------------------------------------------
-// Element-wise kernels around the GEMMs.
+// The network, training and inference.
 namespace sg {
 namespace {
 

@@ -1,6 +1,5 @@
-// Host side of the surrogate: ensemble parameters, training step (captured
-// once as a CUDA graph and replayed), prediction with the acceptance gate,
-// and the C ABI of include/surrogate.h.
+// Host side of the surrogate: ensemble parameters, training steps, prediction
+// with the acceptance gate, and the C ABI of include/surrogate.h.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
