@@ -33,10 +33,10 @@ FALLBACK_HBM_GBS = 6800.0
 # workload, by row chunk, valid only for the sources (kernel_hash) recorded
 # with them.
 NCU_TRAFFIC = {
-    "cfg2": {"kernel_sha": "cf2f590a198bdc85", "bytes_per_step": {80: 721.96e6}},
-    "cfg2h": {"kernel_sha": "cf2f590a198bdc85", "bytes_per_step": {80: 371.28e6}},
-    "cfg4": {"kernel_sha": "96a7e071522f2b2b", "bytes_per_step": {80: 4.6221e9}},
-    "cfg4h": {"kernel_sha": "96a7e071522f2b2b", "bytes_per_step": {80: 2.5061e9}},
+    "cfg2": {"kernel_sha": "96eaa30a3a14ef6f", "bytes_per_step": {80: 722.70e6}},
+    "cfg2h": {"kernel_sha": "96eaa30a3a14ef6f", "bytes_per_step": {80: 369.06e6}},
+    "cfg4": {"kernel_sha": "69e94d85c178f9e0", "bytes_per_step": {56: 4.6286e9}},
+    "cfg4h": {"kernel_sha": "69e94d85c178f9e0", "bytes_per_step": {56: 2.5194e9}},
 }
 
 
