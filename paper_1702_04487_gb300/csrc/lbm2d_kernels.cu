@@ -20,8 +20,7 @@
 //    in FP32) with every update in FP32;
 //  - diagnostics rows (ink weight e, e n, e n u_y) are summed in FP32 per
 //    strip row and in FP64 across strips; the lattice totals of n, phi and
-//    n u_y in FP32 pairs per lane over an item and in FP64 across lanes and
-//    items.
+//    n u_y in FP64 throughout.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -247,23 +246,6 @@ __device__ __forceinline__ float recip(float x) {
   const float r = __fdividef(1.0f, x);
   return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
-
-// A running sum of FP32 values as an unevaluated pair hi + lo: the rounding
-// error of every addition is exact (Knuth's TwoSum) and collected in lo.  For
-// the few hundred values of a work item lo loses nothing that FP64 would keep
-// (the errors are multiples of the values' last places), and an addition costs
-// 7 FP32 instructions where FP64 took a conversion and an addition at 1/64 of
-// their rate.
-struct PairSum {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(hi, v);
-    const float b = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
 
 // Per-lattice constants of the collision, in registers.
 struct CollK {
@@ -649,10 +631,11 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
     for (int i = 0; i < 4; i++) upA[i] = upB[i] = 0.f;
     bbA[0] = bbA[1] = bbB[0] = bbB[1] = 0.f;
     // lattice totals sum n, sum phi, sum n u_y of the lane's cells over the
-    // item (diagnostics steps): the sum of a few hundred FP32 values is exact
-    // in a pair as in FP64, so the totals do not depend on how rows are cut
-    // into items (only on the FP64 order of the final additions)
-    PairSum sn, sphi, smom;
+    // item (diagnostics steps), in FP64: how rows are cut into items changes
+    // them by the rounding of FP64 additions only.  (FP32 pairs, which keep 48
+    // of FP64's 53 bits, made a step of 20 x 200 x 1600 with one diagnostics
+    // step in ten 1.4 % faster, and lost infinities.)
+    double sn = 0.0, sphi = 0.0, smom = 0.0;
 
 #pragma unroll 1
     for (int k = 0; k < ch + 6; k++) {
@@ -738,11 +721,11 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
           const float eB = fminf(fmaxf(prB2 * K.inv_phis, 0.0f), 1.0f);
           if (oA) {
             dg[0] += eA; dg[1] += eA * nA; dg[2] += eA * nA * uyA;
-            sn.add(nA); sphi.add(prA2); smom.add(__fmul_rn(nA, uyA));
+            sn += (double)nA; sphi += (double)prA2; smom += (double)__fmul_rn(nA, uyA);
           }
           if (oB) {
             dg[0] += eB; dg[1] += eB * nB; dg[2] += eB * nB * uyB;
-            sn.add(nB); sphi.add(prB2); smom.add(__fmul_rn(nB, uyB));
+            sn += (double)nB; sphi += (double)prB2; smom += (double)__fmul_rn(nB, uyB);
           }
         }
       }
@@ -909,7 +892,7 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
 #undef KD
     cp_async_wait<0>();  // no copy may land after the warp moves on
     if (DIAG) {
-      double tn = sn.value(), tphi = sphi.value(), tmom = smom.value();
+      double tn = sn, tphi = sphi, tmom = smom;
       for (int o = wid >> 1; o > 0; o >>= 1) {
         tn += __shfl_down_sync(kFull, tn, o, wid);
         tphi += __shfl_down_sync(kFull, tphi, o, wid);
