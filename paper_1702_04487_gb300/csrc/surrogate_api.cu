@@ -84,10 +84,18 @@ struct sg_handle_s {
     void* ptr = nullptr;
     if (alloc)
       ptr = alloc(bytes, ctx);
-    else if (cudaMalloc(&ptr, bytes) != cudaSuccess)
+    else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+      cudaGetLastError();  // reported as IJ_ERR_OOM; the next launch check must not see it
       ptr = nullptr;
+    }
     if (ptr) blocks.push_back(ptr);
     return ptr;
+  }
+  // Give back a block that no launch has used yet (null: nothing).
+  void dfree(void* ptr) {
+    if (!ptr) return;
+    blocks.erase(std::find(blocks.begin(), blocks.end(), ptr));
+    if (free_fn) free_fn(ptr, ctx); else cudaFree(ptr);
   }
   void release() {
     if (stream) cudaStreamSynchronize(stream); else cudaDeviceSynchronize();
@@ -213,12 +221,16 @@ constexpr int kStagedQueries = 1024;
 ij_status ensure_query(sg_handle h, int n) {
   if (n <= h->q_cap) return IJ_OK;
   const size_t nn = (size_t)n, K = h->K;
-  h->q_x = (float*)h->dalloc(nn * kIn * 4);
-  h->q_x16 = (bf16*)h->dalloc(nn * kInPad * 2);
-  h->q_y = (float*)h->dalloc(K * nn * kOut * 4);
-  h->q_out = (float*)h->dalloc((kOutHead + nn * (2 * kOut + 1)) * 4);
-  if (!h->q_x || !h->q_x16 || !h->q_y || !h->q_out)
+  void* b[4] = {h->dalloc(nn * kIn * 4), h->dalloc(nn * kInPad * 2), h->dalloc(K * nn * kOut * 4),
+                h->dalloc((kOutHead + nn * (2 * kOut + 1)) * 4)};
+  if (!b[0] || !b[1] || !b[2] || !b[3]) {
+    for (void* p : b) h->dfree(p);  // the workspace in use stays
     return fail(IJ_ERR_OOM, "device allocation of the query workspace failed");
+  }
+  h->q_x = (float*)b[0];
+  h->q_x16 = (bf16*)b[1];
+  h->q_y = (float*)b[2];
+  h->q_out = (float*)b[3];
   h->q_cap = n;
   return IJ_OK;
 }
@@ -330,13 +342,15 @@ ij_status sg_set_data(sg_handle h, const float* x, const float* y, int n) {
     if (!isfinite(y[i]) || (((h->cfg.log_outputs >> (i % kOut)) & 1) && !(y[i] > 0)))
       return fail(IJ_ERR_PARAM, "outcome row %lld: non-finite or non-positive under a log",
                   i / kOut);
-  fit_xform(x, n, kIn, h->cfg.log_inputs, h->xin);
-  fit_xform(y, n, kOut, h->cfg.log_outputs, h->xout);
+  Xform xin, xout;
+  fit_xform(x, n, kIn, h->cfg.log_inputs, xin);
+  fit_xform(y, n, kOut, h->cfg.log_outputs, xout);
+  float lo[kIn], hi[kIn];
   for (int d = 0; d < kIn; d++) {
-    h->lo[d] = h->hi[d] = x[d];
+    lo[d] = hi[d] = x[d];
     for (int i = 1; i < n; i++) {
-      h->lo[d] = std::min(h->lo[d], x[(size_t)i * kIn + d]);
-      h->hi[d] = std::max(h->hi[d], x[(size_t)i * kIn + d]);
+      lo[d] = std::min(lo[d], x[(size_t)i * kIn + d]);
+      hi[d] = std::max(hi[d], x[(size_t)i * kIn + d]);
     }
   }
   // leave-one-out nearest-neighbour distances in transformed input space
@@ -345,7 +359,7 @@ ij_status sg_set_data(sg_handle h, const float* x, const float* y, int n) {
     for (int d = 0; d < kIn; d++) {
       double v = x[(size_t)i * kIn + d];
       if ((h->cfg.log_inputs >> d) & 1) v = log(v);
-      xt[(size_t)i * kIn + d] = (v - h->xin.mean[d]) / h->xin.scale[d];
+      xt[(size_t)i * kIn + d] = (v - xin.mean[d]) / xin.scale[d];
     }
   std::vector<double> nn(n, 1e300);
   for (int i = 0; i < n; i++)
@@ -359,20 +373,36 @@ ij_status sg_set_data(sg_handle h, const float* x, const float* y, int n) {
       nn[j] = std::min(nn[j], d2);
     }
   std::sort(nn.begin(), nn.end());
-  h->nn_cut = (float)(2.0 * sqrt(nn[(size_t)((n - 1) * 0.95)]));
 
+  // Everything that can run out of memory comes before the handle changes: on
+  // failure the data, transforms and gate it had stay in use.
   cudaStream_t s = h->stream;
+  void *X = nullptr, *T = nullptr, *Xt = nullptr;
+  const int ldt = (n + 127) / 128 * 128;  // the gate reads whole groups of 128 points
+  ij_status st = IJ_OK;
   if (n > h->train_cap) {
-    h->ldt = (n + 127) / 128 * 128;  // the gate reads whole groups of 128 points
-    h->X = (bf16*)h->dalloc((size_t)n * kInPad * 2);
-    h->T = (float*)h->dalloc((size_t)n * kOut * 4);
-    h->Xt = (float*)h->dalloc((size_t)h->ldt * kIn * 4);
-    if (!h->X || !h->T || !h->Xt) return fail(IJ_ERR_OOM, "device allocation of the data failed");
+    X = h->dalloc((size_t)n * kInPad * 2);
+    T = h->dalloc((size_t)n * kOut * 4);
+    Xt = h->dalloc((size_t)ldt * kIn * 4);
+    if (!X || !T || !Xt) st = fail(IJ_ERR_OOM, "device allocation of the data failed");
+  }
+  if (st == IJ_OK) st = ensure_query(h, n);  // raw rows are staged in the query workspace
+  if (st != IJ_OK) {
+    for (void* p : {X, T, Xt}) h->dfree(p);
+    return st;
+  }
+  if (n > h->train_cap) {
+    h->X = (bf16*)X;
+    h->T = (float*)T;
+    h->Xt = (float*)Xt;
+    h->ldt = ldt;
     h->train_cap = n;
   }
-  // raw rows staged in the query workspace
-  ij_status st = ensure_query(h, n);
-  if (st != IJ_OK) return st;
+  h->xin = xin;
+  h->xout = xout;
+  memcpy(h->lo, lo, sizeof(lo));
+  memcpy(h->hi, hi, sizeof(hi));
+  h->nn_cut = (float)(2.0 * sqrt(nn[(size_t)((n - 1) * 0.95)]));
   CUDA_TRY(cudaMemcpyAsync(h->q_x, x, (size_t)n * kIn * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(h->q_out, y, (size_t)n * kOut * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(launch_prep_inputs(h->q_x, n, h->xin, h->X, h->Xt, h->ldt, s));
