@@ -142,6 +142,7 @@ struct ij_handle_s {
     if (alloc) {
       p = alloc(bytes, ctx);
     } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();  // reported as IJ_ERR_OOM; the next launch check must not see it
       p = nullptr;
     }
     if (p) blocks.push_back(p);
@@ -624,6 +625,21 @@ ij_status upload_items(ij_handle h) {
   return IJ_OK;
 }
 
+// Make `want` the buckets of a 2-D handle, with their work list on the device.
+// When the list does not fit, the buckets and the list in use stay.
+ij_status set_buckets(ij_handle h, const std::vector<Bucket>& want) {
+  const std::vector<Bucket> old = h->buckets;
+  const std::vector<Item> items = h->items;
+  h->buckets = want;
+  build_items(h);
+  const ij_status st = upload_items(h);
+  if (st != IJ_OK) {
+    h->buckets = old;
+    h->items = items;
+  }
+  return st;
+}
+
 ij_status check_handle(ij_handle h) {
   if (!h) return fail(IJ_ERR_PARAM, "null handle");
   return IJ_OK;
@@ -753,17 +769,20 @@ ij_status build_graph(ij_handle h) {
 }
 
 // Work items of the 3-D step and their upload (the device array grows only).
-ij_status upload_items3(ij_handle h) {
-  const int n = make_items3(h->inst3.data(), h->n_inst, h->buckets[0].chunk, nullptr);
-  h->items3.resize(n);
-  make_items3(h->inst3.data(), h->n_inst, h->buckets[0].chunk, h->items3.data());
-  if ((size_t)n > h->items3_cap) {
-    h->d_items3 = (Item3*)h->dalloc(n * sizeof(Item3));
-    if (!h->d_items3) return fail(IJ_ERR_OOM, "device allocation of 3-D work items failed");
+ij_status upload_items3(ij_handle h, int chunk) {
+  std::vector<Item3> items(make_items3(h->inst3.data(), h->n_inst, chunk, nullptr));
+  const size_t n = items.size();
+  make_items3(h->inst3.data(), h->n_inst, chunk, items.data());
+  if (n > h->items3_cap) {
+    Item3* p = (Item3*)h->dalloc(n * sizeof(Item3));
+    if (!p) return fail(IJ_ERR_OOM, "device allocation of 3-D work items failed");
+    h->d_items3 = p;  // the old list stays owned by the handle until destroy
     h->items3_cap = n;
   }
+  h->items3.swap(items);
   Bucket& b = h->buckets[0];
-  b.count = n;
+  b.chunk = chunk;
+  b.count = (int)n;
   CUDA_TRY(cudaMemcpyAsync(h->d_items3, h->items3.data(), n * sizeof(Item3), cudaMemcpyHostToDevice,
                            h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -896,7 +915,7 @@ ij_status create3(ij_handle h) {
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   h->buckets.assign(1, Bucket{kStep3Threads, 0, 0, sms, default_chunk3(h->inst3, sms), 1, false, 0});
-  ij_status st = upload_items3(h);
+  ij_status st = upload_items3(h, h->buckets[0].chunk);
   if (st != IJ_OK) return st;
   cudaStream_t s = h->stream;
   CUDA_TRY(cudaMemcpyAsync(h->d_inst3, h->inst3.data(), count * sizeof(Inst3), cudaMemcpyHostToDevice, s));
@@ -925,8 +944,9 @@ ij_status create3(ij_handle h) {
 // FP32 staging buffer for exporting / importing a lattice's state (3-D, 2-D FP16).
 ij_status ensure_stage(ij_handle h, size_t floats) {
   if (h->stage_floats >= floats) return IJ_OK;
-  h->stage = (float*)h->dalloc(floats * sizeof(float));
-  if (!h->stage) return fail(IJ_ERR_OOM, "device allocation of the staging buffer failed");
+  float* p = (float*)h->dalloc(floats * sizeof(float));
+  if (!p) return fail(IJ_ERR_OOM, "device allocation of the staging buffer failed");
+  h->stage = p;
   h->stage_floats = floats;
   return IJ_OK;
 }
@@ -1323,27 +1343,23 @@ ij_status ij_tune(ij_handle h, int block_size, int chunk, int prefetch) {
     // the z chunk of the 3-D work items; one block size, no prefetch depth
     if (chunk < 1 || prefetch != 1 || (block_size > 0 && block_size != kStep3Threads))
       return fail(IJ_ERR_PARAM, "3-D handles take chunk >= 1, prefetch 1, block size %d", kStep3Threads);
-    h->buckets[0].chunk = chunk;
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    return upload_items3(h);
+    return upload_items3(h, chunk);
   }
   if (chunk < -5 || prefetch < 1 || prefetch > kMaxPrefetch)
     return fail(IJ_ERR_PARAM, "chunk must be >= -5 and prefetch in 1..%d", kMaxPrefetch);
   bool found = false;
-  for (Bucket& b : h->buckets)
+  std::vector<Bucket> want = h->buckets;
+  for (Bucket& b : want)
     if (block_size <= 0 || b.nthreads == block_size) {
       found = true;
-    }
-  for (Bucket& b : h->buckets)
-    if (block_size <= 0 || b.nthreads == block_size) {
       b.chunk = chunk;
       b.prefetch = prefetch;
       b.cells = false;
     }
   if (!found) return fail(IJ_ERR_PARAM, "no lattice of the handle runs with %d threads", block_size);
   CUDA_TRY(cudaStreamSynchronize(h->stream));
-  build_items(h);
-  return upload_items(h);
+  return set_buckets(h, want);
 }
 
 }  // extern "C"
@@ -1365,12 +1381,12 @@ ij_status autotune3(ij_handle h, int reps) {
   CUDA_TRY(cudaEventCreate(&e0));
   CUDA_TRY(cudaEventCreate(&e1));
   float best = 1e30f;
-  int best_chunk = h->buckets[0].chunk;
+  const int old_chunk = h->buckets[0].chunk;
+  int best_chunk = old_chunk;
   ij_status st = IJ_OK;
   for (int chunk : kChunks3) {
     if (chunk > 2 * max_nz) continue;
-    h->buckets[0].chunk = chunk;
-    st = upload_items3(h);
+    st = upload_items3(h, chunk);
     if (st != IJ_OK) break;
     const int n = (int)h->items3.size();
     cudaError_t e = launch_step3(h->d_inst3, h->d_items3, n, h->n_inst, h->d_t, 0, false, h->fp16,
@@ -1394,9 +1410,9 @@ ij_status autotune3(ij_handle h, int reps) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (st == IJ_ERR_OOM) upload_items3(h, old_chunk);  // fits: it was there
   if (st != IJ_OK) return st;
-  h->buckets[0].chunk = best_chunk;
-  return upload_items3(h);
+  return upload_items3(h, best_chunk);
 }
 
 }  // namespace
@@ -1415,6 +1431,7 @@ ij_status ij_autotune(ij_handle h, int reps) {
   cudaEvent_t e0, e1;
   CUDA_TRY(cudaEventCreate(&e0));
   CUDA_TRY(cudaEventCreate(&e1));
+  const std::vector<Bucket> old = h->buckets;
   // Trial launches read the state at t and write only the other time buffer
   // (without diagnostics), so the state is unchanged; t does not advance.
   for (size_t bi = 0; bi < h->buckets.size(); bi++) {
@@ -1430,12 +1447,17 @@ ij_status ij_autotune(ij_handle h, int reps) {
       for (int chunk : kChunks) {
         if (chunk > 2 * max_ny && chunk > 0) continue;
         if (pf == 0 && chunk != kChunks[0]) continue;
-        h->buckets[bi].cells = pf == 0;
-        h->buckets[bi].chunk = pf ? chunk : best_chunk;
-        h->buckets[bi].prefetch = pf ? pf : best_pf;
-        build_items(h);
-        st = upload_items(h);
-        if (st != IJ_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+        std::vector<Bucket> want = h->buckets;
+        want[bi].cells = pf == 0;
+        want[bi].chunk = pf ? chunk : best_chunk;
+        want[bi].prefetch = pf ? pf : best_pf;
+        st = set_buckets(h, want);
+        if (st != IJ_OK) {
+          cudaEventDestroy(e0);
+          cudaEventDestroy(e1);
+          if (st == IJ_ERR_OOM) set_buckets(h, old);  // fits: it was there
+          return st;
+        }
         const Bucket& b = h->buckets[bi];
         CUDA_TRY(launch_bucket(h, b, 0, false, h->stream));  // warm-up
         CUDA_TRY(cudaEventRecord(e0, h->stream));
@@ -1453,14 +1475,16 @@ ij_status ij_autotune(ij_handle h, int reps) {
           best_pf = b.prefetch;
         }
       }
-    h->buckets[bi].cells = best_cells;
-    h->buckets[bi].chunk = best_chunk;
-    h->buckets[bi].prefetch = best_pf;
+    std::vector<Bucket> want = h->buckets;
+    want[bi].cells = best_cells;
+    want[bi].chunk = best_chunk;
+    want[bi].prefetch = best_pf;
+    st = set_buckets(h, want);  // fits: it was timed
+    if (st != IJ_OK) break;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  build_items(h);
-  return upload_items(h);
+  return st;
 }
 
 ij_status ij_use_graph(ij_handle h, int enable) {

@@ -86,3 +86,41 @@ def test_training_data_that_do_not_fit(allocator, left):
         assert np.array_equal(a, b)
     sg.set_data(*more)  # it fits again
     assert np.isfinite(sg.predict(more[0])[0]).all()
+
+
+def _states(ij, h, n):
+    return [u for k in range(n) for u in ij.ij_get_state(h, k)]
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_work_lists_that_do_not_fit(allocator, dim):
+    """A longer work list that cannot be uploaded leaves the list in use."""
+    from paper_1702_04487_gb300 import inkjet as ij, workloads as W
+    p = W.small_nozzle(nx=70, ny=4000) if dim == 2 else W.small_nozzle3(nx=64, ny=64, nz=160)
+    h, twin = ij.ij_create(p), ij.ij_create(p)
+    for s in (h, twin):
+        ij.ij_tune(s, 0, 64, 1)
+    before = ij.ij_get_tuning(h)
+    _refused(allocator, 0, lambda: ij.ij_tune(h, 0, 1, 1))
+    assert ij.ij_get_tuning(h) == before
+    _refused(allocator, 0, lambda: ij.ij_autotune(h, 1))
+    assert ij.ij_get_tuning(h) == before
+    for s in (h, twin):
+        ij.ij_step(s, 25)
+    for a, b in zip(_states(ij, h, 1), _states(ij, twin, 1)):
+        assert np.array_equal(a, b)
+    ij.ij_tune(h, 0, 1, 1)  # it fits again
+    ij.ij_step(h, 1)
+
+
+def test_states_that_do_not_fit(allocator):
+    """The FP32 staging buffer of FP16 and 3-D states grows with the lattice."""
+    from paper_1702_04487_gb300 import inkjet as ij, workloads as W
+    for ps in ([W.small_nozzle(precision=1), W.small_nozzle(nx=96, ny=160, precision=1)],
+               [W.small_nozzle3(), W.small_nozzle3(nx=30, ny=30)]):
+        h = ij.ij_create(ps)
+        want = ij.ij_get_state(h, 0)
+        _refused(allocator, 0, lambda: ij.ij_get_state(h, 1))
+        for a, b in zip(ij.ij_get_state(h, 0), want):
+            assert np.array_equal(a, b)
+        assert all(np.isfinite(u).all() for u in ij.ij_get_state(h, 1))
