@@ -212,7 +212,7 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  * columns on each side), times a range of rows of one lattice, with the
  * populations staged `prefetch` rows (1..4) ahead of use; every block is
  * one warp (32 threads), so a finished item frees its slot at once.  Every
- * lattice of a handle is in the one bucket of 32-thread blocks.  The work
+ * lattice of a handle is in its one bucket.  The work
  * list comes in two forms, chosen by `chunk`:
  *   chunk >= 1 : rows cut into chunks of `chunk` rows; the list starts with
  *                the rows of nozzle-wall strips below the nozzle exit
@@ -230,18 +230,21 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  * An untuned handle takes -1 while its lattices give each item only a few
  * rows, and beyond that the row chunk (8 .. 56) whose list makes one to three
  * waves of items.  Up to 240000 cells, its steps without diagnostics run a
- * kernel with a block per 16 x 8 tile of cells instead of the list
- * (ij_autotune times it as one more candidate, ij_tune turns it off).
+ * kernel with a block of 192 threads per 16 x 8 tile of cells instead of the
+ * list (ij_autotune times it as one more candidate).
  *
- * ij_tune      -- set chunk (>= -5) and prefetch (block_size: 32, or <= 0
- *                 for every bucket).  Synchronises.
+ * ij_tune      -- set chunk (>= -5) and prefetch.  block_size 32, or <= 0 for
+ *                 every bucket: every step runs the list; 192, up to 240000
+ *                 cells: steps without diagnostics run the tile kernel, the
+ *                 others the list.  Synchronises.
  * ij_autotune  -- time `reps` trial launches of every candidate (chunks
  *                 8..128 in steps of 8, 160, 192, 256 and 0 .. -5; prefetch
  *                 1..4) on the current state
  *                 and keep the fastest.  Trial launches leave the state and
  *                 the time unchanged.  Synchronises.
- * ij_get_tuning -- block size, chunk, prefetch and item count of bucket
- *                 `bucket` (0-based); IJ_ERR_PARAM past the last bucket.
+ * ij_get_tuning -- block size (192 with the tile kernel, else 32), chunk,
+ *                 prefetch and item count of bucket `bucket` (0-based), which
+ *                 ij_tune takes as they are; IJ_ERR_PARAM past the last bucket.
  * 3-D handles have one bucket of 512-thread blocks (one CTA per 28 x 12
  * column tile and z chunk); its one tunable is the z chunk: ij_tune takes
  * chunk >= 1 and prefetch 1 (block_size 512 or <= 0), ij_autotune times

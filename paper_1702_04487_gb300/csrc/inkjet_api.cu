@@ -1348,14 +1348,18 @@ ij_status ij_tune(ij_handle h, int block_size, int chunk, int prefetch) {
   }
   if (chunk < -5 || prefetch < 1 || prefetch > kMaxPrefetch)
     return fail(IJ_ERR_PARAM, "chunk must be >= -5 and prefetch in 1..%d", kMaxPrefetch);
+  // the block size of the kernel of small lattices asks for that kernel, where
+  // an untuned handle would take it, so that what ij_get_tuning reports gives
+  // another handle the same kernels
+  const bool cells = block_size == kCellThreads && default_cells(h);
   bool found = false;
   std::vector<Bucket> want = h->buckets;
   for (Bucket& b : want)
-    if (block_size <= 0 || b.nthreads == block_size) {
+    if (block_size <= 0 || b.nthreads == block_size || cells) {
       found = true;
       b.chunk = chunk;
       b.prefetch = prefetch;
-      b.cells = false;
+      b.cells = cells;
     }
   if (!found) return fail(IJ_ERR_PARAM, "no lattice of the handle runs with %d threads", block_size);
   CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -1500,7 +1504,7 @@ ij_status ij_get_tuning(ij_handle h, int bucket, int* block_size, int* chunk, in
   if (st != IJ_OK) return st;
   if (bucket < 0 || bucket >= (int)h->buckets.size()) return fail(IJ_ERR_PARAM, "no such bucket");
   const Bucket& b = h->buckets[bucket];
-  if (block_size) *block_size = b.nthreads;
+  if (block_size) *block_size = b.cells ? kCellThreads : b.nthreads;
   if (chunk) *chunk = b.chunk;
   if (prefetch) *prefetch = b.prefetch;
   if (items) *items = b.count;

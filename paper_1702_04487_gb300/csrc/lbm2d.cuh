@@ -59,6 +59,7 @@ struct Item {
 constexpr int kStripCols = 60;     // written columns of one work item
 constexpr long long kCellsMost = 240000;  // cells of a handle or call that take launch_cells
 constexpr int kStepThreads = 32;  // one warp per block, one work item each
+constexpr int kCellThreads = 192;  // threads of a block of the kernel of small lattices
 constexpr int kStepBlocksPerSM = 10;  // resident blocks per SM the registers are sized for
 constexpr int kMaxPrefetch = 4;    // rows staged ahead of use: 1 .. 4
 

@@ -926,7 +926,6 @@ __global__ void __launch_bounds__(32, kStepBlocksPerSM)
 constexpr int kCellX = 16, kCellY = 8;
 constexpr int kCellRX = kCellX + 6, kCellRY = kCellY + 6;  // phi: three rings
 constexpr int kCellCX = kCellX + 2, kCellCY = kCellY + 2;  // colliding cells
-constexpr int kCellThreads = 192;
 static_assert(kCellCX * kCellCY <= kCellThreads, "a thread per colliding cell");
 
 // ONE: a handle of one lattice, whose descriptor comes with the launch and
