@@ -1449,8 +1449,7 @@ ij_status ij_autotune(ij_handle h, int reps) {
     const bool try_cells = default_cells(h);  // one more candidate: pf 0, no list
     for (int pf = try_cells ? 0 : 1; pf <= kMaxPrefetch; pf++)
       for (int chunk : kChunks) {
-        if (chunk > 2 * max_ny && chunk > 0) continue;
-        if (pf == 0 && chunk != kChunks[0]) continue;
+        if (pf == 0 ? chunk != kChunks[0] : chunk > 2 * max_ny) continue;
         std::vector<Bucket> want = h->buckets;
         want[bi].cells = pf == 0;
         want[bi].chunk = pf ? chunk : best_chunk;

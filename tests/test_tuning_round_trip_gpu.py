@@ -66,3 +66,15 @@ def test_tiles_are_refused_where_an_untuned_handle_does_not_take_them(ij):
             ij.ij_tune(h, size, 24, 1)
         assert e.value.status == ij.IJ_ERR_PARAM
     assert ij.ij_get_tuning(h) == before
+
+
+@pytest.mark.parametrize("nx,ny", [(2000, 3), (64, 1), (64, 5), (64, 256)])
+def test_autotune_times_the_tiles_of_every_small_lattice(ij, nx, ny):
+    """Four prefetch depths of each list, and the tiles once, however few the
+    rows (a candidate is a warm-up and one timed launch)."""
+    from paper_1702_04487_gb300 import workloads as W
+    h = ij.ij_create(dict(W.small_nozzle(nx=nx, ny=ny, F0=1e-4, F_neg=5e-5), geometry=0))
+    n = ij.ij_launch_count(h)
+    ij.ij_autotune(h, 1)
+    candidates = (ij.ij_launch_count(h) - n) // 2
+    assert candidates % 4 == 1
