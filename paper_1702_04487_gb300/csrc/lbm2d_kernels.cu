@@ -1648,7 +1648,15 @@ int make_items(const Inst& I, int k, int chunk, Item* out, int cap) {
 }
 
 int items_per_range(const Inst& I, int chunk, int ya, int yb, bool allow_half) {
-  return yb > ya ? make_items_range(I, 0, chunk, ya, yb, nullptr, 0, allow_half) : 0;
+  if (yb <= ya) return 0;
+  const int rows = yb - ya, nstrip = (I.nx + kStripCols - 1) / kStripCols;
+  const int last = I.nx - (nstrip - 1) * kStripCols;
+  const bool half = allow_half && last <= kStripCols / 2 - 2;
+  const int per_strip = (rows + chunk - 1) / chunk;
+  if (!half) return nstrip * per_strip;
+  // pairs of whole chunks, then what is left chunk by chunk (strip_items)
+  const int pairs = rows / chunk / 2;
+  return (nstrip - 1) * per_strip + pairs + (rows - 2 * pairs * chunk + chunk - 1) / chunk;
 }
 
 int items_per_lattice(const Inst& I, int chunk) { return items_per_range(I, chunk, 0, I.ny, true); }
