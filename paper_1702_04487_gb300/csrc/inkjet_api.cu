@@ -873,7 +873,6 @@ ij_status create3(ij_handle h) {
   if (e3 != cudaSuccess) return fail(IJ_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e3));
   h->inst3.resize(count);
   h->inst.resize(count);
-  std::vector<int2> ghosts;
   for (int k = 0; k < count; k++) {
     const ij_params& p = h->params[k];
     Inst3 I = derive3(p);
@@ -888,14 +887,13 @@ ij_status create3(ij_handle h) {
       if (!I.f[b] || !I.g[b] || !I.g0[b] || !I.phi[b])
         return fail(IJ_ERR_OOM, "device allocation of 3-D lattice %d failed", k);
     }
-    I.n_ghost = derived_phi3(I, nullptr);
-    ghosts.resize(std::max(1, I.n_ghost));
-    derived_phi3(I, ghosts.data());
+    const std::vector<int2> ghosts = derived_phi3(I);
+    I.n_ghost = (int)ghosts.size();
     I.ghost = (int2*)h->dalloc(ghosts.size() * sizeof(int2));
     if (!I.ghost) return fail(IJ_ERR_OOM, "device allocation of 3-D lattice %d failed", k);
     CUDA_TRY(cudaMemcpyAsync(I.ghost, ghosts.data(), ghosts.size() * sizeof(int2),
                              cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));  // ghosts is reused
+    CUDA_TRY(cudaStreamSynchronize(h->stream));  // ghosts goes out of scope
     // the step never stores solid cells: they hold 0 in both buffers
     for (int b = 0; b < 2; b++) {
       CUDA_TRY(cudaMemsetAsync(I.f[b], 0, std::max(19 * N * es, N * sizeof(double)), h->stream));

@@ -4,6 +4,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "lbm2d.cuh"
 
 namespace ij {
@@ -55,9 +57,8 @@ struct Item3 {
 constexpr int kTile3X = 28, kTile3Y = 12;  // written columns of a 3-D work item
 constexpr int kStep3Threads = 512;          // threads of a step3 CTA (32 x 16 columns)
 
-// The derived entries of phi (Inst3::ghost), written to out when not null;
-// returns their number.  Host code.
-int derived_phi3(const Inst3& h, int2* out);
+// The derived entries of phi (Inst3::ghost).  Host code.
+std::vector<int2> derived_phi3(const Inst3& h);
 // Work items of every lattice into out (null: count only); returns the count.
 int make_items3(const Inst3* h, int n_inst, int chunk, Item3* out);
 

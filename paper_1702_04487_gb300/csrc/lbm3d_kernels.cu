@@ -1012,29 +1012,74 @@ dim3 grid3(const Inst3& h) { return dim3((h.nx + 31) / 32, (h.ny + 3) / 4, h.nz)
 
 }  // namespace
 
-int derived_phi3(const Inst3& h, int2* out) {
-  int cnt = 0;
-  auto add = [&](int x, int y, int z, bool all) {
-    const int kind = kind_at3(h, x, y, z);
-    unsigned m = kind == 0 ? kGhostCopy : (kind == 2 ? kGhostWet : 0u);
-    if (kind != 0)
-      for (int i = 1; i < 19; i++)
-        if (kind_at3(h, x + ex3(i), y + ey3(i), z + ez3(i)) == 0) m |= 1u << (i - 1);
-    if (!all && !(m & 0x3FFFFu)) return;  // out of reach of every fluid stencil
-    if (out) out[cnt] = make_int2(((z + 2) * h.ny + y) * h.nx + x, (int)m);
-    cnt++;
+// The geometry has at most four kinds of plane: fluid, outside a closed end,
+// the walls of the nozzle (or the plate's body), the plate's top.  What a plane
+// adds to the list follows from its kind and those of its two neighbours, so
+// each such triple is worked out once, over bytes, and copied for every plane
+// that has it.  Evaluating the geometry of 18 neighbours of every solid cell
+// took half of ij_create (64 lattices of 20 x 20 x 64: 33 ms).
+std::vector<int2> derived_phi3(const Inst3& h) {
+  enum { kFluid, kOutside, kBody, kTop, kKinds };
+  const int nx = h.nx, ny = h.ny, plane = nx * ny;
+  const int solid = h.geom == GEOM_NOZZLE ? h.L : h.geom == GEOM_PLATE ? h.wt : 0;
+  const int zmax = std::min(solid, h.nz);  // planes with solid cells
+  auto plane_of = [&](int z) {
+    int zm;
+    if (!map_z(h, z, zm)) return (int)kOutside;
+    if (zm >= solid) return (int)kFluid;
+    return (int)(h.geom == GEOM_PLATE && zm == solid - 1 ? kTop : kBody);
   };
-  int zmax = 0;
-  if (h.geom == GEOM_NOZZLE) zmax = std::min(h.L, h.nz);
-  if (h.geom == GEOM_PLATE) zmax = std::min(h.wt, h.nz);
-  for (int z = 0; z < zmax; z++)
-    for (int y = 0; y < h.ny; y++)
-      for (int x = 0; x < h.nx; x++)
-        if (geom_kind3(h, x, y, z) != 0) add(x, y, z, false);
-  for (int z : {-2, -1, h.nz, h.nz + 1})
-    for (int y = 0; y < h.ny; y++)
-      for (int x = 0; x < h.nx; x++) add(x, y, z, true);
-  return cnt;
+  // cell kinds (0 fluid, 1 solid, 2 solid on a wetting face) of each plane
+  std::vector<unsigned char> kinds[kKinds];
+  kinds[kFluid].assign(plane, 0);
+  kinds[kOutside].assign(plane, 1);
+  for (int k : {kBody, kTop}) {
+    kinds[k].resize(plane);
+    for (int y = 0; y < ny; y++)
+      for (int x = 0; x < nx; x++)
+        kinds[k][y * nx + x] =
+            solid > 0 ? (unsigned char)geom_kind3(h, x, y, k == kTop ? solid - 1 : 0) : 0;
+  }
+  // the entries {cell of the plane, mask} of a plane between two others: every
+  // point (for an extended plane), and the solid cells that a fluid stencil
+  // reaches (for a plane of the lattice)
+  int dx[19], dy[19], dz[19];
+  for (int i = 1; i < 19; i++) {
+    dx[i] = 1 + ex3(i);
+    dy[i] = 1 + ey3(i);
+    dz[i] = 1 + ez3(i);
+  }
+  struct Entries { std::vector<int2> all, reached; } made[kKinds * kKinds * kKinds];
+  auto entries = [&](int z) -> const Entries& {
+    const int k3[3] = {plane_of(z - 1), plane_of(z), plane_of(z + 1)};
+    Entries& list = made[(k3[0] * kKinds + k3[1]) * kKinds + k3[2]];
+    if (!list.all.empty()) return list;
+    list.all.reserve(plane);
+    for (int y = 0; y < ny; y++) {
+      const unsigned char* row[3][3];  // of the three planes, at y - 1 .. y + 1
+      for (int j = 0; j < 9; j++)
+        row[j / 3][j % 3] = kinds[k3[j / 3]].data() + wrap3(y - 1 + j % 3, ny) * nx;
+      for (int x = 0; x < nx; x++) {
+        const int kind = row[1][1][x];
+        unsigned m = kind == 0 ? kGhostCopy : (kind == 2 ? kGhostWet : 0u);
+        if (kind != 0) {
+          const int xs[3] = {wrap3(x - 1, nx), x, wrap3(x + 1, nx)};
+          for (int i = 1; i < 19; i++)
+            m |= (unsigned)(row[dz[i]][dy[i]][xs[dx[i]]] == 0) << (i - 1);
+        }
+        list.all.push_back(make_int2(y * nx + x, (int)m));
+        if (kind != 0 && (m & 0x3FFFFu)) list.reached.push_back(list.all.back());
+      }
+    }
+    return list;
+  };
+  std::vector<int2> out;
+  auto add = [&](int z, const std::vector<int2>& list) {
+    for (const int2& e : list) out.push_back(make_int2((z + 2) * plane + e.x, e.y));
+  };
+  for (int z = 0; z < zmax; z++) add(z, entries(z).reached);
+  for (int z : {-2, -1, h.nz, h.nz + 1}) add(z, entries(z).all);
+  return out;
 }
 
 // Tiles of 28 x 12 columns, z chunks of `chunk` planes; a z chunk of every
