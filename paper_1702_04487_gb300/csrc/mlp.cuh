@@ -96,6 +96,9 @@ cudaError_t launch_schedule_begin(const long long* d_step, long long* d_sched, l
 // BF16 copies of the parameters without an update.
 cudaError_t launch_cast_params(const float* p, const Layout& L, int members, bf16* Wb, bf16* WbT,
                                cudaStream_t s);
+// Allow the network's kernels (training and inference) their shared memory on
+// the current device: called for each handle that is made, on its device.
+cudaError_t allow_network_smem();
 // Outputs of every member for n raw queries x [n][7]: Y [m][n][4] (FP32,
 // transformed outcomes).  One kernel runs all five layers of a 128-row tile.
 cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* p, const bf16* Wb,

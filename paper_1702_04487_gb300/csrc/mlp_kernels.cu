@@ -337,18 +337,24 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 // The driver's tensor-map encoder, looked up once through the runtime (no
 // link against the driver library).
 EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  static bool looked = false;
-  if (!looked) {
-    looked = true;
+  // (the initialisation of a local static is safe with several threads)
+  static const EncodeTiledFn fn = []() -> EncodeTiledFn {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
                                          &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+      return reinterpret_cast<EncodeTiledFn>(p);
+    return nullptr;
+  }();
   return fn;
+}
+
+// Dynamic shared memory beyond 48 KB has to be allowed for a kernel, on each
+// device: nothing about it is kept between calls.
+template <typename F>
+cudaError_t allow_smem(F* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // 3-D tensor map of a BF16 operand: K (contiguous) x rows (leading dimension
@@ -376,14 +382,8 @@ cudaError_t launch_bn(const GemmArgs& a, cudaStream_t s) {
   CUtensorMap ma, mb;
   cudaError_t e0 = make_map(&ma, a.A, a.K, a.M, a.lda, 0, 1, BM);
   if (e0 == cudaSuccess) e0 = make_map(&mb, a.B, a.K, a.N, a.ldb, 0, 1, BN);
+  if (e0 == cudaSuccess) e0 = allow_smem(gemm_kernel<BN>, smem);
   if (e0 != cudaSuccess) return e0;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   dim3 grid((a.M + BM - 1) / BM, (a.N + BN - 1) / BN);
   gemm_kernel<BN><<<grid, kThreads, smem, s>>>(ma, mb, a);
   return cudaGetLastError();
@@ -1340,6 +1340,7 @@ __global__ void __launch_bounds__(kChainThreads, 1)
 // copy and a counter launch took 85 us.
 constexpr int kUpdateThreads = 512;
 constexpr int kUpdateBN = 64;
+constexpr size_t kUpdateSmem = kStages * (size_t)stage_bytes<kUpdateBN>() + kFwdTail;
 
 struct UpdateMaps {
   CUtensorMap a[kHidden + 1];  // dZ_l^T, boxes of 64 (rows of the minibatch) x 128
@@ -1702,13 +1703,6 @@ __global__ void advance_step_kernel(long long* d_step, int by) { *d_step += by; 
 template <bool TRAIN>
 cudaError_t launch_chain(const ChainMaps& maps, const ChainArgs& a, int members, cudaStream_t s) {
   const int ctas = chain_ctas(a.H);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(chain_kernel<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)chain_smem_bytes(256));
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks(a.rows, BM) * ctas, members);
   cfg.blockDim = dim3(kChainThreads);
@@ -1739,6 +1733,15 @@ cudaError_t chain_maps(ChainMaps* m, const Layout& L, int members, const bf16* W
 }
 
 }  // namespace
+
+cudaError_t allow_network_smem() {
+  cudaError_t e = allow_smem(chain_kernel<true>, chain_smem_bytes(256));
+  if (e == cudaSuccess) e = allow_smem(chain_kernel<false>, chain_smem_bytes(256));
+  if (e == cudaSuccess) e = allow_smem(forward_kernel, fwd_smem_bytes(256, kFwdRing));
+  if (e == cudaSuccess) e = allow_smem(pair_kernel, pair_smem_bytes(256));
+  if (e == cudaSuccess) e = allow_smem(update_kernel, kUpdateSmem);
+  return e;
+}
 
 cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* p, const bf16* Wb,
                            const Layout& L, int members, float* Y, unsigned* status,
@@ -1778,16 +1781,6 @@ cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* 
     cudaError_t e = make_map(&maps.w[l], Wb + L.w_off[l], L.nin[l], L.nout[l], L.nin[l], L.total,
                              members, 128);
     if (e != cudaSuccess) return e;
-  }
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fwd_smem_bytes(256, kFwdRing));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)pair_smem_bytes(256));
-    if (e != cudaSuccess) return e;
-    attr = true;
   }
   if ((long long)grid.x * grid.y <= 152)  // at most one tile per SM
     forward_kernel<<<grid, kFwdThreads, fwd_smem_bytes(a.H, kFwdRing), s>>>(maps, a);
@@ -1855,17 +1848,10 @@ cudaError_t launch_train_step(const TrainArgs& t, cudaStream_t s) {
       e = make_map(&um.b[l], B, t.rows, nb, t.rows, (long long)nb * t.rows, t.members, kUpdateBN);
     if (e != cudaSuccess) return e;
   }
-  static bool attr = false;
-  const size_t smem = kStages * (size_t)stage_bytes<kUpdateBN>() + kFwdTail;
-  if (!attr) {
-    e = cudaFuncSetAttribute(update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(u.first[kHidden + 1], t.members);
   cfg.blockDim = dim3(kUpdateThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = kUpdateSmem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

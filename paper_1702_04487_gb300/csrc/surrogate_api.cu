@@ -298,6 +298,8 @@ ij_status sg_create(const sg_config* cfg, ij_alloc_fn alloc, ij_free_fn free_fn,
     if (!b) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
   for (int l = 0; l < kHidden; l++)
     if (!h->Ht[l] || !h->dZt[l]) return bail(fail(IJ_ERR_OOM, "device allocation failed"));
+  const cudaError_t e = allow_network_smem();
+  if (e != cudaSuccess) return bail(fail(IJ_ERR_CUDA, "allow_network_smem: %s", cudaGetErrorString(e)));
   // He-uniform initialisation on the host (once), zero biases and padding
   std::vector<float> init(KP, 0.0f);
   for (int mem = 0; mem < h->K; mem++)
