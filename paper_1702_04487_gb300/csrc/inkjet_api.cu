@@ -521,26 +521,34 @@ int chunk_items(const Inst& I, int chunk) {
 
 // The chunk of a handle that is not tuned, from its warp rows (strip rows, a
 // half-warp strip counting half) per work item that the GPU runs at once
-// (152 SMs x 12).  Figures: us a step, in brackets with the 7/8 + tail list
-// (0) that every untuned handle took before.
-//  - Few rows per slot (under 12; 30 with one or two lattices; 50 while
-//    lattices have at most four strips, none of them narrow): equal pieces
-//    making one wave (-1).  What runs together then fits in L2 or lies close
-//    together, and an even end matters more than the order of the items:
-//    200 x 1600 16.8 (22.5), 57 x 98 x 229 40.3 (44.8), 1000 x 3000 70.3
-//    (72.7), 17 x 240 x 812 67.9 (72.6, and 81.9 in 32-row chunks).  At most
-//    four whole strips keep list 0 up to 250 rows per slot: 80 x 100 x 1000
-//    191, 218 in row chunks.
-//  - Beyond, row chunks, neighbouring rows of neighbouring strips together,
-//    whose halo reads meet in L2 and whose DRAM pages are shared: the chunk
-//    that makes about 2300 items, one wave and its short last pieces, up to
-//    40 rows per slot of equal lattices or 20 of uneven ones (8 x 200 x 1600
-//    61.5 (71.6), 10 uneven of 1.3 M cells 39.6 (43.3)), about 5000 items
-//    above, 56 rows and an eighth of the height at most (61 x 184 x 456 133
-//    (144), 20 x 200 x 1600 153 (188), 256 uneven lattices of 34.6 M cells
-//    770 (1090)).
-// Over 44 drawn sets of 0.9 to 28 M cells the choice is within 2 % of the best
-// chunk on the average and 1.12 x faster than list 0 (0.98 x at worst).
+// (152 SMs x 12).  The candidates: equal pieces making one wave (-1), whose
+// even end matters most while there are few rows per slot; the same with a tail
+// of short pieces (0, what every untuned handle took at first); row chunks,
+// neighbouring rows of neighbouring strips together, whose halo reads meet in L2
+// and whose DRAM pages are shared.  Balanced pieces keep no half-warp items, so
+// row chunks also serve lattices that end on a narrow strip.  The lines lie
+// where the better side changes over 1681 drawn sets of 0.25 to 30 M cells (up to
+// 300 lattices, FP32 and FP16, equal and uneven, a record every ten steps; us a
+// step, the choice first):
+//  - under 12 rows per slot, 30 with one or two lattices: -1 (200 x 1600 16.8,
+//    22.5 with 0; 17 x 51 x 55 7.1, 12.2);
+//  - at most four whole strips: -1 up to 50 rows, 0 up to 250 (80 x 100 x 1000
+//    191, 218 in row chunks);
+//  - hardly any narrow strips (under 5 % more warp rows for whole warps): -1 up
+//    to 60 rows in FP16 storage, whose steps are bound by issue and gain little
+//    from shared pages (6 x 1950 x 366 78, 94 in row chunks), 30 in FP32 from 10
+//    strips on and 40 from 25, where a wave of pieces already lies side by side
+//    (2000 x 2000 87, 96 in row chunks; 7 x 342 x 1092, 6 strips: 67 and 62.5);
+//  - lattices of under 100 rows (200 if they differ), whose chunks would be
+//    shorter than their 6 pipeline rows pay for: -1 up to 20 rows, 0 up to 60
+//    (80 x 382 x 66 57.6, 65.4 in row chunks);
+//  - row chunks beyond: the chunk that makes about 2300 items, one wave and its
+//    short last pieces, up to 40 rows per slot of equal lattices or 20 of uneven
+//    ones (8 x 200 x 1600 61.5, 71.6 with 0), about 5000 items above, 56 rows and
+//    an eighth of the height at most (20 x 200 x 1600 153 (188), 256 uneven
+//    lattices of 34.6 M cells 770 (1090)).
+// Over 723 further sets the choice takes 0.896 of list 0's time and 1.027 of the
+// best candidate's; one set in twelve is more than 2 % slower than list 0.
 int default_chunk(ij_handle h, const Bucket& b) {
   double rows = 0.0, full = 0.0;  // full: a whole warp for every strip
   int strips = 0, ny = 1;
@@ -555,9 +563,15 @@ int default_chunk(ij_handle h, const Bucket& b) {
     equal = equal && I.nx == h->inst[0].nx && I.ny == h->inst[0].ny;
   }
   const double per_slot = rows / std::max(1, step_slots(b.prefetch, h->fp16, h->odd));
-  const bool narrow = full > 1.02 * rows;
+  const double narrow = full / rows;  // 1: no strip is narrow
   if (per_slot < 12.0 || (h->n_inst <= 2 && per_slot <= 30.0)) return -1;
-  if (strips <= 4 && !narrow && per_slot <= 250.0) return per_slot <= 50.0 ? -1 : 0;
+  if (strips <= 4 && narrow <= 1.02 && per_slot <= 250.0) return per_slot <= 50.0 ? -1 : 0;
+  const double even = h->fp16 ? 60.0 : strips >= 25 ? 40.0 : strips >= 10 ? 30.0 : 12.0;
+  if (narrow <= 1.05 && per_slot < even) return -1;
+  if (equal ? ny < 100 && narrow <= 1.1 : ny < 200) {
+    if (per_slot < 20.0) return -1;
+    if (per_slot < 60.0) return 0;
+  }
   constexpr int kLongest = 56;
   if (per_slot > 200.0) return kLongest;
   const int want = per_slot < (equal ? 40.0 : 20.0) ? 2300 : 5000;
