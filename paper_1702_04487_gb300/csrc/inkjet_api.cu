@@ -1,6 +1,7 @@
 // Host side of libinkjet.so: parameter validation and derivation, device
 // memory, work lists and launches of the 2-D step (include/inkjet.h).
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -831,19 +832,21 @@ ij_status upload_items3(ij_handle h, int chunk) {
   return IJ_OK;
 }
 
-// The z chunk of a 3-D handle that is not tuned: the one whose busiest CTA
-// marches over the fewest planes (each item takes its planes and about three
-// more: two re-read at its ends, and the start of its pipeline), weighted by
-// 1 + 0.0006 chunk because longer chunks keep fewer neighbouring tiles in step
-// and so lose halo reads in L2.  Measured (us a step) at the choice, against
-// the 80 planes that every lattice took before: 32 x 32 x 160 45.5 (8 planes)
-// and 235, 64 x 64 x 320 142 (40) and 246, 100 x 80 x 300 226 (64) and 270;
-// 2 x 128 x 128 x 640 keeps 80.
+// The z chunk of a 3-D handle that is not tuned: the one whose busiest CTA has
+// the fewest planes to do, an item counting four more than it writes (two
+// re-read at its ends, the start and end of its pipeline); the shorter chunk on
+// a tie.  Over 744 drawn sets (24 .. 200 cells across, up to 640 planes, 1 .. 24
+// lattices, both storages) the choice is 0.08 % above the best of 15 chunks on
+// the average and never more than 0.5 % slower than the 80 planes that every
+// lattice took at first, whose time it halves: 32 x 32 x 160 31 us a step with 7
+// planes (198 with 80), 64 x 64 x 320 118 with 40 (211), 100 x 80 x 300 186 with 30
+// (220); 2 x 128 x 128 x 640 keeps 80.  With three planes an item and a weight of
+// 1 + 0.0006 chunk, ten sets were 2 to 5.5 % slower than with 80 planes.
 int default_chunk3(const std::vector<Inst3>& inst, int ctas) {
   static const int kTry[] = {1,  2,  3,  4,  5,  6,  7,  8,  9,  10, 11, 12, 13, 14, 15,  16,  18,
                              20, 22, 24, 26, 28, 30, 32, 36, 40, 44, 48, 56, 64, 72, 80, 96, 128};
-  int best = 80;
-  double best_cost = 1e300;
+  constexpr int kItemPlanes = 4;
+  int best = 80, best_cost = INT_MAX;
   std::vector<int> load;
   for (int chunk : kTry) {
     // items in the order of make_items3, item k on CTA k mod ctas
@@ -859,11 +862,11 @@ int default_chunk3(const std::vector<Inst3>& inst, int ctas) {
         const int ch = std::min(chunk, I.nz - z0);
         const int whole = tiles / (int)load.size();
         if (whole)
-          for (int& v : load) v += whole * (ch + 3);
-        for (int j = 0; j < tiles % (int)load.size(); j++) load[(k + j) % load.size()] += ch + 3;
+          for (int& v : load) v += whole * (ch + kItemPlanes);
+        for (int j = 0; j < tiles % (int)load.size(); j++) load[(k + j) % load.size()] += ch + kItemPlanes;
         k += tiles;
       }
-    const double cost = *std::max_element(load.begin(), load.end()) * (1.0 + 0.0006 * chunk);
+    const int cost = *std::max_element(load.begin(), load.end());
     if (cost < best_cost) {
       best_cost = cost;
       best = chunk;
