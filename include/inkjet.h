@@ -212,8 +212,8 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  * columns on each side), times a range of rows of one lattice, with the
  * populations staged `prefetch` rows (1..4) ahead of use; every block is
  * one warp (32 threads), so a finished item frees its slot at once.  Every
- * lattice of a handle is in its one bucket.  The work
- * list comes in two forms, chosen by `chunk`:
+ * lattice of a handle is in its one bucket.  The work list comes in two forms,
+ * chosen by `chunk`:
  *   chunk >= 1 : rows cut into chunks of `chunk` rows; the list starts with
  *                the rows of nozzle-wall strips below the nozzle exit
  *                (costlier per row) and ends with the last eighth of each
@@ -228,10 +228,11 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  *                3, 4 full waves.
  *
  * An untuned handle takes -1 while its lattices give each item only a few
- * rows, and beyond that the row chunk (8 .. 56) whose list makes one to three
- * waves of items.  Up to 240000 cells, its steps without diagnostics run a
- * kernel with a block of 192 threads per 16 x 8 tile of cells instead of the
- * list (ij_autotune times it as one more candidate).
+ * rows, and beyond that -1, 0 or the row chunk (8 .. 56) whose list makes one to
+ * three waves of items, by the number, sizes and storage of its lattices.  Up
+ * to 240000 cells, its steps without diagnostics run a kernel with a block of
+ * 192 threads per 16 x 8 tile of cells instead of the list (ij_autotune times it
+ * as one more candidate).
  *
  * ij_tune      -- set chunk (>= -5) and prefetch.  block_size 32, or <= 0 for
  *                 every bucket: every step runs the list; 192, up to 240000
@@ -249,7 +250,8 @@ ij_status ij_kernel_timing(ij_handle h, int enable, double* total_ms, long long*
  * column tile and z chunk); its one tunable is the z chunk: ij_tune takes
  * chunk >= 1 and prefetch 1 (block_size 512 or <= 0), ij_autotune times
  * chunks of 8 .. 256 planes and the untuned choice (the chunk whose busiest
- * CTA has the fewest planes).  Results do not depend on the chunk.
+ * CTA has the fewest planes, an item counting four more than it writes).
+ * Results do not depend on the chunk.
  */
 ij_status ij_tune(ij_handle h, int block_size, int chunk, int prefetch);
 /* ij_use_graph -- run whole diagnostics periods (diag_every steps, or 16
@@ -297,8 +299,10 @@ ij_status ij_get_tuning(ij_handle h, int bucket, int* block_size, int* chunk, in
  * on a device looks up that array's device address, so make it before any
  * stream capture.  Every call shares the array: calls whose GPU work
  * overlaps (for example on two streams) race, so order them on one stream.
- * The descriptor, the time and the work list are copied from static host
- * buffers with cudaMemcpyAsync under a mutex (no host heap either).
+ * Up to 240000 cells without record_out the descriptor and the time come with
+ * the launch, and only the flag is written to the array (without status_out);
+ * otherwise they and the work list are copied from static host buffers with
+ * cudaMemcpyAsync.  Either way under a mutex and without the host heap.
  * Errors: IJ_ERR_PARAM, IJ_ERR_CUDA.
  */
 ij_status ij_step_noalloc(const ij_params* params, long long t, const float* f_in,

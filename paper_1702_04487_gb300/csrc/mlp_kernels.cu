@@ -499,7 +499,9 @@ __global__ void cast_params_kernel(const float* __restrict__ p, const Layout L, 
 // tensor-memory lanes 32 (w mod 4) .. + 31 and every (warps / 4)-th group of
 // 16 units.
 //
-// Bound by latency here (up to a tile per SM); many tiles take pair_kernel.
+// Bound by latency (a tile per SM at most; many tiles take pair_kernel): five
+// members of H = 256, queries and answers on the device, take 82 us a call from
+// 385 to 3072 queries.
 constexpr int kFwdChunk = 128 * BK * 2;  // bytes of a weight chunk, and of 64 activation columns
 constexpr int kFwdRing = 9;
 
@@ -519,8 +521,7 @@ struct FwdArgs {
 
 constexpr int kFwdThreads = 512;
 // activations, ring, then the barriers and the tensor-memory address (no
-// static shared memory: the dynamic part then starts on a 1024-byte boundary
-// and two CTAs of H = 256 fit an SM)
+// static shared memory: the dynamic part then starts on a 1024-byte boundary)
 constexpr int kFwdTail = 256;
 size_t fwd_smem_bytes(int H, int ring) {
   return (size_t)((H + BK - 1) / BK + ring) * kFwdChunk + kFwdTail;
@@ -1750,7 +1751,12 @@ cudaError_t launch_forward(const float* x, int n, const Xform& xf, const float* 
   const dim3 grid(blocks(n, BM), members);
   if ((long long)grid.x * grid.y * chain_ctas(L.nout[0]) <= 152) {
     // few tiles: a cluster per tile splits the layers (up to 384 queries of
-    // five members of H = 256; a call of one query 49 us, 74 with a CTA per tile)
+    // five members of H = 256; a call of one query 49 us, 74 with a CTA per
+    // tile).  Up to 152 CTAs: not all of the largest clusters run at once then,
+    // but two waves of them still take no longer than a CTA per tile (queries
+    // on the device, H = 256: three members 67 us up to 120 CTAs, 80 with 144,
+    // 82 with a CTA per tile; one member 78 with 128 and 152 CTAs, 81; eight
+    // members 80 with 128, 84)
     ChainMaps cm = {};
     cudaError_t e = chain_maps(&cm, L, members, Wb, nullptr);
     if (e != cudaSuccess) return e;
