@@ -33,10 +33,10 @@ FALLBACK_HBM_GBS = 6800.0
 # workload, by row chunk, valid only for the sources (kernel_hash) recorded
 # with them.
 NCU_TRAFFIC = {
-    "cfg2": {"kernel_sha": "96eaa30a3a14ef6f", "bytes_per_step": {80: 722.70e6}},
-    "cfg2h": {"kernel_sha": "96eaa30a3a14ef6f", "bytes_per_step": {80: 369.06e6}},
-    "cfg4": {"kernel_sha": "69e94d85c178f9e0", "bytes_per_step": {56: 4.6286e9}},
-    "cfg4h": {"kernel_sha": "69e94d85c178f9e0", "bytes_per_step": {56: 2.5194e9}},
+    "cfg2": {"kernel_sha": "7642ac3c486ad060", "bytes_per_step": {80: 722.86e6}},
+    "cfg2h": {"kernel_sha": "7642ac3c486ad060", "bytes_per_step": {80: 369.28e6}},
+    "cfg4": {"kernel_sha": "f8c2a11c7b77c3d1", "bytes_per_step": {80: 4.6206e9}},
+    "cfg4h": {"kernel_sha": "f8c2a11c7b77c3d1", "bytes_per_step": {80: 2.5175e9}},
 }
 
 
